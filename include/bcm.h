@@ -115,9 +115,12 @@ typedef struct {
                                  one per wave of sources (ceil(n / lanes)).  Each holds a slot of
                                  44 E lanes/64 bytes, E its table's entries (cta_table); with the
                                  one-source kernel (BCM_SPARSE) 8 ceil(n/32) + 16 Q bytes, Q =
-                                 min(n, 2^18) where an overflowing source can be deferred, else n */
+                                 min(n, 2^18) where an overflowing source can be deferred, else n;
+                                 on undirected graphs of largest degree <= 8 (padded rows) 8 Q, and
+                                 ceil(n/32) words more above 1.6 M vertices */
     uint32_t threads;         /* threads per CTA of the per-CTA kernel: 256, 512 or 1024; 0 = 512
-                                 (the one-source kernel, BCM_SPARSE: also 128; 0 = 256) */
+                                 (the one-source kernel, BCM_SPARSE: also 128; 0 = 256, on padded
+                                 rows a choice by n) */
     uint32_t heavy_words;     /* see above; 0 = default (4 per warp of the grid) */
     uint32_t pull_div;        /* a grid-wave level is expanded by pull when the out-arcs of its
                                  frontier's (vertex, word) entries number at least n*W/pull_div
@@ -167,7 +170,8 @@ typedef struct {
                                  started, 28 per frontier word, 12 per (arc, frontier word), 32 per
                                  new frontier word, 28 per cleared word; the one-source kernel: 20 per
                                  source, 12 per frontier vertex, 8 per arc, 16 per discovered vertex,
-                                 12 per cleared bitmap word */
+                                 12 per cleared bitmap word (padded rows: 20 per source and 4 per row
+                                 entry of a frontier vertex, the rest is in shared memory) */
     uint64_t grid_waves;      /* waves run by the grid-wide kernel */
     uint64_t grid_levels;     /* levels those waves expanded */
     uint64_t grid_bytes;      /* algorithmic bytes of the grid-wide kernel (same unit costs) */

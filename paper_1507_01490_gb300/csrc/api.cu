@@ -58,9 +58,9 @@ static bcm_status cuda_fail(cudaError_t e, const char* what) {
 // of one layout overlap the bit arrays of another.
 struct Layout {
     uint32_t n = 0, W = 0, blocks = 0, entries = 0;   // entries: the vertex tables', or the sparse queues'
-    bool sparse = false;
+    int kind = 0;   // 0 waves, 1 one source per CTA, 2 the same on a padded adjacency
     bool operator==(const Layout& o) const {
-        return n == o.n && W == o.W && blocks == o.blocks && entries == o.entries && sparse == o.sparse;
+        return n == o.n && W == o.W && blocks == o.blocks && entries == o.entries && kind == o.kind;
     }
 };
 struct Region { int dev; void* ptr; size_t bytes; Layout layout; };
@@ -333,6 +333,7 @@ struct bcm_graph {
                                    // level 1 of every BFS is then known from degrees alone (the prefilter)
     bool preprocessed = false;
     uint32_t max_deg = 0;          // largest row length (found by preprocessing)
+    uint32_t* d_lat = nullptr;     // padded adjacency of k_lattice, laid out by the first run that needs it
     Aux* d_aux = nullptr;
     uint32_t* d_plain = nullptr;   // stamps [n], two vertex queues [2n]
     unsigned long long* d_far = nullptr;   // exhaustive outputs [n]
@@ -344,7 +345,8 @@ struct bcm_graph {
         bool active = false;
         bool exhaustive = false;
         bool plain = false;
-        bool sparse = false;      // the per-CTA phase ran k_sparse
+        bool sparse = false;      // the per-CTA phase ran one source per CTA
+        int lat = 0;              // ... on the padded adjacency of this many entries per row
         uint32_t kk = 0;          // entries the top-k must hold
         uint32_t flags = 0;
         uint64_t l0 = 0;          // launch counter at the start
@@ -385,6 +387,7 @@ struct Cfg {
     uint32_t cta_entries, tab_shift;   // per-CTA vertex tables (WaveParams)
     bool sparse;                       // per-CTA phase: one source per CTA (k_sparse)
     uint32_t sparse_qcap;
+    int lat;                           // ... by k_lattice, rows of this many entries (0: k_sparse)
 };
 
 // Entries of a hashed per-CTA vertex table by default: n/8 rounded up to a
@@ -430,12 +433,14 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
     c->sparse = !(o.flags & BCM_GRID_ONLY) &&
                 ((o.flags & BCM_SPARSE) || (!(o.flags & BCM_NO_SPARSE) && !g->directed && g->n >= 4096 &&
                                             g->max_deg <= kSparseMaxDeg));
-    // its default block is 256 threads: on damaged grids 512 threads took
+    // on undirected graphs whose rows fit the padded adjacency: k_lattice
+    c->lat = !c->sparse || g->directed || g->n > (1u << 28) ? 0 : g->max_deg <= 4 ? 4 : g->max_deg <= 8 ? 8 : 0;
+    // k_sparse's default block is 256 threads: on damaged grids 512 threads took
     // 3.4 s against 2.5 s at 512^2, 128 threads 25.7 s against 23.6 s at
     // 1024^2 (it also runs 128)
-    c->threads = o.threads ? (int)o.threads : (c->sparse ? 256 : 512);
+    c->threads = o.threads ? (int)o.threads : (c->lat ? lattice_threads(g->n) : c->sparse ? 256 : 512);
     if (c->sparse) {
-        if (c->threads != 128 && c->threads != 256 && c->threads != 512 && c->threads != 1024)
+        if (o.threads && o.threads != 128 && o.threads != 256 && o.threads != 512 && o.threads != 1024)
             return fail(BCM_ERR_UNSUPPORTED, "threads must be 128, 256, 512 or 1024 (got %u)", o.threads);
     } else {
         if (c->threads != 256 && c->threads != 512 && c->threads != 1024)
@@ -483,7 +488,7 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
     const bool sparse_defer = !(c->flags & (BCM_CTA_ONLY | BCM_GRID_ONLY)) && c->defer_words;
     c->sparse_qcap = (sparse_defer && g->n > kSparseQcap) ? kSparseQcap : g->n;
     if (c->sparse) {
-        const int sper = sparse_blocks_per_sm(c->threads);
+        const int sper = c->lat ? lattice_blocks_per_sm(g->n, c->threads, c->lat) : sparse_blocks_per_sm(c->threads);
         if (sper < 1) return fail(BCM_ERR_CUDA, "one-source kernel does not fit on an SM");
         const int smax = sper * g->sms;
         c->blocks = o.blocks ? (int)o.blocks : (g->n < (uint32_t)smax ? (int)(g->n ? g->n : 1) : smax);
@@ -500,7 +505,8 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
 
 // CTA slots first, then one slot (4 words per vertex) for the grid-wide waves.
 size_t cta_slot_stride(bcm_graph* g, const Cfg& c) {
-    return c.sparse ? sparse_slot_bytes(g->n, c.sparse_qcap) : slot_bytes(c.cta_entries, c.W);
+    return c.lat ? lattice_slot_bytes(g->n, c.sparse_qcap)
+           : c.sparse ? sparse_slot_bytes(g->n, c.sparse_qcap) : slot_bytes(c.cta_entries, c.W);
 }
 size_t cta_region_bytes(bcm_graph* g, const Cfg& c) { return (size_t)c.blocks * cta_slot_stride(g, c); }
 size_t region_bytes(bcm_graph* g, const Cfg& c) {
@@ -512,7 +518,7 @@ Layout region_layout(bcm_graph* g, const Cfg& c) {
     l.W = (uint32_t)c.W;
     l.blocks = (uint32_t)c.blocks;
     l.entries = c.sparse ? c.sparse_qcap : c.cta_entries;
-    l.sparse = c.sparse;
+    l.kind = c.lat ? 2 : c.sparse ? 1 : 0;
     return l;
 }
 
@@ -719,6 +725,7 @@ WaveParams base_params(bcm_graph* g, const Cfg& c) {
     p.slot_base = (char*)g->slots.ptr;
     p.slot_stride = cta_slot_stride(g, c);
     p.sparse_qcap = c.sparse_qcap;
+    p.lat_rows = g->d_lat;
     p.cta_entries = c.cta_entries;
     p.tab_shift = c.tab_shift;
     p.tab_limit = c.cta_entries / 2;
@@ -761,6 +768,13 @@ uint64_t wave_alg_bytes(const unsigned long long* w, uint64_t sources) {
 uint64_t sparse_alg_bytes(const unsigned long long* w, uint64_t sources) {
     return 20ull * sources + 12ull * w[ST_ENTRIES] + 8ull * w[ST_ARCWORDS] + 16ull * w[ST_DISCWORDS] +
            12ull * w[ST_CLEARED];
+}
+
+// k_lattice's (its bitmap and its queues' first entries lie in shared memory):
+//   source started            20 B  order entry, row_ptr pair, x_lo
+//   frontier vertex expanded  4 B per entry of its padded row
+uint64_t lattice_alg_bytes(const unsigned long long* w, uint64_t sources, int rw) {
+    return 20ull * sources + 4ull * rw * w[ST_ENTRIES];
 }
 
 void fill_stats(bcm_stats* s, const unsigned long long* st, uint64_t launches, double kms, double pms, double tms) {
@@ -850,6 +864,11 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     if ((st = ensure_run_state(g, trace))) return st;
     const bool plain = !exhaustive && (c.flags & BCM_PLAIN);
     if (!plain && (st = ensure_slots(g, c))) return st;
+    if (!plain && c.lat && !g->d_lat) {
+        CU(buf_get_t(&g->d_lat, (size_t)g->n * c.lat * sizeof(uint32_t)), "padded adjacency allocation");
+        if (launch_lattice_rows(g->d_rp, g->d_col, g->n, c.lat, g->d_lat, s))
+            return fail(BCM_ERR_CUDA, "padded adjacency kernel: %s", cudaGetErrorString(cudaGetLastError()));
+    }
     if (exhaustive && !g->d_far) {
         CU(buf_get_t(&g->d_far, (size_t)g->n * sizeof(uint64_t) + 256), "output allocation");
         CU(buf_get_t(&g->d_reach, (size_t)g->n * sizeof(uint32_t) + 256), "output allocation");
@@ -966,7 +985,9 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
             pc.n_end_dev = &g->d_aux->surv_n;
         }
         if (rc == 0)
-            rc = c.sparse ? launch_sparse(pc, c.blocks, c.threads, s) : launch_cta_waves(pc, c.W, c.blocks, c.threads, s);
+            rc = c.lat      ? launch_lattice(pc, c.lat, c.blocks, c.threads, s)
+                 : c.sparse ? launch_sparse(pc, c.blocks, c.threads, s)
+                            : launch_cta_waves(pc, c.W, c.blocks, c.threads, s);
         cudaEventRecord(g->ev[2], s);
         if (defer && rc == 0) {
             // the deferred sources, on the grid kernel, every wave
@@ -1011,6 +1032,7 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     g->pend.exhaustive = exhaustive;
     g->pend.plain = plain;
     g->pend.sparse = !plain && c.sparse;
+    g->pend.lat = plain ? 0 : c.lat;
     g->pend.kk = k < n_src ? k : n_src;
     g->pend.flags = c.flags;
     return BCM_OK;
@@ -1074,6 +1096,7 @@ void fill_run_stats(bcm_stats* stats, bcm_graph* g, const unsigned long long* sv
     stats->seed_ms = rt.seed_ms;
     stats->wave_ms = rt.wave_ms;
     stats->wave_bytes = plain ? 0
+                      : g->pend.lat    ? lattice_alg_bytes(wv, wv[ST_WAVES], g->pend.lat)
                       : g->pend.sparse ? sparse_alg_bytes(wv, wv[ST_WAVES])
                                        : wave_alg_bytes(wv, wv[ST_COMPLETED] + wv[ST_CUT]);
     stats->sparse = g->pend.sparse ? wv[ST_WAVES] : 0;
@@ -1213,7 +1236,7 @@ bcm_status bcm_graph_destroy(bcm_graph_t g) {
     else cudaDeviceSynchronize();
     for (void* b : {(void*)g->d_rp, (void*)g->d_col, (void*)g->d_order, (void*)g->d_aux, (void*)g->d_plain,
                     (void*)g->d_far, (void*)g->d_reach, (void*)g->d_rrp, (void*)g->d_rcol, (void*)g->d_trace,
-                    (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv})
+                    (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lat})
         buf_put(b);
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -1294,6 +1317,7 @@ bcm_status bcm_topk_start(bcm_graph_t g, uint32_t k, const bcm_options* opt, uin
         g->pend.exhaustive = false;
         g->pend.plain = false;
         g->pend.sparse = false;
+        g->pend.lat = 0;
         g->pend.kk = 0;
         g->pend.flags = 0;
     }
@@ -1650,7 +1674,7 @@ uint64_t bcm_workspace_bytes(bcm_graph_t g, const bcm_options* opt) {
     if (!g->preprocessed && preprocess(g, nullptr) != BCM_OK) return 0;   // the default kernels depend on it
     Cfg c;
     if (resolve(g, opt, &c)) return 0;
-    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * 12;
+    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * (12 + 4 * c.lat);
 }
 
 }  // extern "C"

@@ -96,6 +96,7 @@ struct WaveParams {
     // one-source-per-CTA kernel: entries of each vertex queue (a longer
     // frontier defers the source)
     uint32_t sparse_qcap;
+    const uint32_t* lat_rows;   // k_lattice: the padded adjacency (launch_lattice_rows)
     char* seed_base;         // the grid kernel's own slot (4 words per vertex)
     unsigned long long* stats;   // [ST_COUNT]
     int* err;
@@ -190,6 +191,15 @@ int cta_blocks_per_sm(int W, int threads);
 // one source per CTA (high-diameter graphs): sources p.sources[*p.head .. n_end)
 int launch_sparse(const WaveParams& p, int blocks, int threads, cudaStream_t s);
 int sparse_blocks_per_sm(int threads);
+
+// ---- lattice.cu: one source per CTA on a padded adjacency of rw = 4 or 8 entries per vertex
+// (undirected graphs of largest degree <= rw, n <= 2^28)
+int launch_lattice_rows(const uint32_t* rp, const uint32_t* col, uint32_t n, int rw, uint32_t* rows, cudaStream_t s);
+int launch_lattice(const WaveParams& p, int rw, int blocks, int threads, cudaStream_t s);
+int lattice_threads(uint32_t n);
+int lattice_blocks_per_sm(uint32_t n, int threads, int rw);
+bool lattice_smem(uint32_t n);   // its visited bitmap lies in shared memory
+size_t lattice_slot_bytes(uint32_t n, uint32_t qcap);
 
 // launch bookkeeping (api.cu)
 void note_launch(int count = 1);
