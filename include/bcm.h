@@ -77,7 +77,8 @@ typedef enum {
 #define BCM_NO_DEFER      0x200u /* per-CTA waves never hand their sources to the grid-wide pass */
 #define BCM_NO_PREFILTER  0x400u /* no level-0/1 prefilter before the per-CTA waves (it runs on simple
                                     graphs -- sorted rows, no repeated arc, no self-loop -- after the
-                                    grid-wide waves; results are the same) */
+                                    grid-wide waves; results are the same); no landmark bounds before
+                                    the searches of large undirected graphs of largest degree <= 8 */
 #define BCM_NO_CUT        0x800u /* bcm_topk: no source is ever stopped by the bound, every BFS runs to its
                                     end (Algorithm 1 without BFSCut is the textbook algorithm of Section
                                     2.1); the top-k is the same -- a check of the cut, not a fast path */

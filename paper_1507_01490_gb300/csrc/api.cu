@@ -334,6 +334,7 @@ struct bcm_graph {
     bool preprocessed = false;
     uint32_t max_deg = 0;          // largest row length (found by preprocessing)
     uint32_t* d_lat = nullptr;     // padded adjacency of k_lattice, laid out by the first run that needs it
+    char* d_lm = nullptr;          // landmark bounds' working memory (landmark.cu)
     Aux* d_aux = nullptr;
     uint32_t* d_plain = nullptr;   // stamps [n], two vertex queues [2n]
     unsigned long long* d_far = nullptr;   // exhaustive outputs [n]
@@ -388,6 +389,7 @@ struct Cfg {
     bool sparse;                       // per-CTA phase: one source per CTA (k_sparse)
     uint32_t sparse_qcap;
     int lat;                           // ... by k_lattice, rows of this many entries (0: k_sparse)
+    bool landmarks;                    // ... with landmark bounds before the searches (top-k runs)
 };
 
 // Entries of a hashed per-CTA vertex table by default: n/8 rounded up to a
@@ -418,6 +420,12 @@ constexpr uint32_t kSparseMaxDeg = 8;
 // deferred to the grid-wide pass (else n).
 constexpr uint32_t kSparseQcap = 1u << 18;
 
+// Landmark bounds from this many vertices on: below it their four BFS, one
+// after another, take longer than the searches that they save (damaged grids,
+// without / with: 64^2 0.77 / 0.89 ms, 100 x 50 0.44 / 0.82, 90^2 1.80 /
+// 1.17, 128^2 4.95 / 1.63).
+constexpr uint32_t kLandmarkMinN = 8192;
+
 bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
     bcm_options o{};
     if (opt) o = *opt;
@@ -435,6 +443,8 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
                                             g->max_deg <= kSparseMaxDeg));
     // on undirected graphs whose rows fit the padded adjacency: k_lattice
     c->lat = !c->sparse || g->directed || g->n > (1u << 28) ? 0 : g->max_deg <= 4 ? 4 : g->max_deg <= 8 ? 8 : 0;
+    c->landmarks = c->lat && g->n >= kLandmarkMinN &&
+                   !(o.flags & (BCM_NO_PREFILTER | BCM_NO_CUT | BCM_TRACE_LANES | BCM_PLAIN));
     // k_sparse's default block is 256 threads: on damaged grids 512 threads took
     // 3.4 s against 2.5 s at 512^2, 128 threads 25.7 s against 23.6 s at
     // 1024^2 (it also runs 128)
@@ -984,6 +994,28 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
             pc.n_end = 0;
             pc.n_end_dev = &g->d_aux->surv_n;
         }
+        if (rc == 0 && c.landmarks && !exhaustive) {
+            // sources by landmark bound; the most central ones first, which
+            // sets the threshold; the others if no bound stops them
+            if (!g->d_lm) {
+                cudaError_t e = buf_get_t(&g->d_lm, landmark_bytes(g->n));
+                if (e != cudaSuccess) { cudaStreamSynchronize(s); return cuda_fail(e, "landmark allocation"); }
+            }
+            const Landmarks L = landmark_carve(g->d_lm, g->n);
+            uint32_t* order = nullptr;
+            rc = launch_landmarks(pc, L, c.lat, n_src, &order, s);
+            uint32_t seeds = (uint32_t)g->sms > 2 * k ? (uint32_t)g->sms : 2 * k;
+            seeds = seeds < n_src ? seeds : n_src;
+            pc.sources = order;
+            pc.n_end = seeds;
+            if (rc == 0) rc = launch_lattice(pc, c.lat, (int)seeds < c.blocks ? (int)seeds : c.blocks, c.threads, s);
+            if (rc == 0) rc = launch_landmark_filter(pc, L, order, seeds, n_src, s);
+            pc.sources = L.list_b;
+            pc.head = &g->d_aux->head3;
+            pc.n_end = 0;
+            pc.n_end_dev = &L.info->n_b;
+            pc.lat_lb = L.lb;
+        }
         if (rc == 0)
             rc = c.lat      ? launch_lattice(pc, c.lat, c.blocks, c.threads, s)
                  : c.sparse ? launch_sparse(pc, c.blocks, c.threads, s)
@@ -1236,7 +1268,7 @@ bcm_status bcm_graph_destroy(bcm_graph_t g) {
     else cudaDeviceSynchronize();
     for (void* b : {(void*)g->d_rp, (void*)g->d_col, (void*)g->d_order, (void*)g->d_aux, (void*)g->d_plain,
                     (void*)g->d_far, (void*)g->d_reach, (void*)g->d_rrp, (void*)g->d_rcol, (void*)g->d_trace,
-                    (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lat})
+                    (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lat, (void*)g->d_lm})
         buf_put(b);
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -1461,8 +1493,9 @@ bcm_status bcm_graph_trim(bcm_graph_t g) {
     CU(g->stream ? cudaStreamSynchronize(g->stream) : cudaDeviceSynchronize(), "synchronize");
     region_release(g->slots, true);
     for (void* b : {(void*)g->d_plain, (void*)g->d_far, (void*)g->d_reach, (void*)g->d_trace, (void*)g->d_defer,
-                    (void*)g->d_shard, (void*)g->d_surv})
+                    (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lm})
         buf_put(b);
+    g->d_lm = nullptr;
     g->d_surv = nullptr;
     g->d_defer = nullptr;
     g->d_shard = nullptr;
@@ -1674,7 +1707,8 @@ uint64_t bcm_workspace_bytes(bcm_graph_t g, const bcm_options* opt) {
     if (!g->preprocessed && preprocess(g, nullptr) != BCM_OK) return 0;   // the default kernels depend on it
     Cfg c;
     if (resolve(g, opt, &c)) return 0;
-    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * (12 + 4 * c.lat);
+    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * (12 + 4 * c.lat) +
+           (c.landmarks ? landmark_bytes(g->n) : 0);
 }
 
 }  // extern "C"

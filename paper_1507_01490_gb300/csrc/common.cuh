@@ -124,6 +124,14 @@ __device__ __forceinline__ bool bfscut_stops(u64 f_d, u64 g, u32 d, u32 n_d, u32
     return all_strict || (all_weak && v > t.id);
 }
 
+// The same rule for any lower bound lb on f(v), r(v) = x known.
+__device__ __forceinline__ bool bound_stops(u64 lb, u32 x, u32 v, const ThrCache& t) {
+    if (!t.valid) return false;
+    const unsigned __int128 xm1 = x - 1;
+    const unsigned __int128 lhs = (unsigned __int128)lb * t.N, rhs = (unsigned __int128)t.F * xm1 * xm1;
+    return lhs > rhs || (lhs == rhs && v > t.id);
+}
+
 // ------------------------------------------------------- shared top-k
 struct TopK {
     u32* id;          // [k] rank order, best first

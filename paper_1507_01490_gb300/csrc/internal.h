@@ -97,6 +97,7 @@ struct WaveParams {
     // frontier defers the source)
     uint32_t sparse_qcap;
     const uint32_t* lat_rows;   // k_lattice: the padded adjacency (launch_lattice_rows)
+    const unsigned long long* lat_lb;   // k_lattice: per vertex, a lower bound on its farness (NULL: none)
     char* seed_base;         // the grid kernel's own slot (4 words per vertex)
     unsigned long long* stats;   // [ST_COUNT]
     int* err;
@@ -200,6 +201,35 @@ int lattice_threads(uint32_t n);
 int lattice_blocks_per_sm(uint32_t n, int threads, int rw);
 bool lattice_smem(uint32_t n);   // its visited bitmap lies in shared memory
 size_t lattice_slot_bytes(uint32_t n, uint32_t qcap);
+// Landmark bounds for k_lattice's sources (landmark.cu).  Working memory, carved out of one block of
+// landmark_bytes(n):
+struct Landmarks {
+    float4* dist;                    // [n] distances from the four landmarks (all ones: not in their component)
+    uint32_t* mind;                  // [n] distance to the nearest landmark so far
+    uint32_t* lv_cnt;                // [4][n + 1] vertices within a distance of landmark i
+    unsigned long long* lv_sum;      // [4][n + 1] their distance sum
+    uint32_t* queue;                 // [2][n] BFS queues past the part in shared memory
+    uint32_t* bitmap;                // [n bits] where shared memory is too small
+    unsigned long long* lb;          // [n] the best bound on f(v) known
+    unsigned long long* joint;       // [n] the joint bound (k_lm_joint)
+    unsigned long long* sample;      // [kLmSample] the joint bound of sampled sources
+    uint32_t *key, *key_tmp, *val, *val_tmp;   // [n] sources by bound
+    uint32_t *list_a, *list_b;       // [n] sources left after the one-landmark / the joint bound
+    void* radix;
+    struct Info {
+        uint32_t size, valid;        // of the landmarks' component; 0: distances too large, no bound
+        uint32_t levels[4];
+        uint32_t n_a, n_b, go;       // list lengths; the joint bound is worth taking
+    }* info;
+};
+size_t landmark_bytes(uint32_t n);
+Landmarks landmark_carve(void* base, uint32_t n);
+// distances and one-landmark bounds; *order gets the n_src sources p.sources[0..) by ascending bound
+int launch_landmarks(const WaveParams& p, const Landmarks& L, int rw, uint32_t n_src, uint32_t** order, cudaStream_t s);
+// sources order[first..n_src) that no bound stops -> L.list_b, their count in L.info->n_b; the others
+// are counted as cut
+int launch_landmark_filter(const WaveParams& p, const Landmarks& L, const uint32_t* order, uint32_t first,
+                           uint32_t n_src, cudaStream_t s);
 
 // launch bookkeeping (api.cu)
 void note_launch(int count = 1);

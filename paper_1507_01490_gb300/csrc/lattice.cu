@@ -26,17 +26,15 @@
 // ms, 512^2 1,534 -> 389 ms, 1/16 of 1024^2's sources 1.47 s -> 0.73 s.
 #include <cuda_runtime.h>
 
-#include "internal.h"
+#include "lattice.cuh"
 #include "trace.cuh"
 
 namespace bcm {
 
 constexpr u32 kLatQueue = 1024;          // queue entries in shared memory, per queue
-constexpr u32 kLatSmemMaxN = 1600000;    // bitmap in shared memory up to this n (200 KB)
 // Threads an SM holds at once (the register budget): 48 registers for rows of
 // 4.  512^2: 389 ms; 1536 threads (40 registers, spills) 439, 1024 400.
 constexpr int kLatResident = 1280;
-constexpr u32 kLatIdMask = 0x0fffffffu;  // neighbour id; the degree is above it
 
 bool lattice_smem(uint32_t n) { return n <= kLatSmemMaxN; }
 
@@ -109,29 +107,12 @@ __device__ __noinline__ void lattice_complete(const WaveParams& p, ThrCache& t, 
     lock_release(p.topk.lock);
 }
 
-// Sets `bit` of a bitmap word where `seen` says that it was clear, and
-// returns the word as it was (all ones where nothing was done): predicated
-// by hand, since the compiler branches around each of a row's atomics.
-template <bool SMEM>
-__device__ __forceinline__ u32 set_if_clear(u32* word, u32 bit, u32 seen) {
-    u32 old = ~0u;
-    if (SMEM) {
-        const u32 at = (u32)__cvta_generic_to_shared(word);
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %3, 0;\n\t@p atom.shared.or.b32 %0, [%1], %2;\n\t}"
-                     : "+r"(old) : "r"(at), "r"(bit), "r"(seen) : "memory");
-    } else {
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %3, 0;\n\t@p atom.global.or.b32 %0, [%1], %2;\n\t}"
-                     : "+r"(old) : "l"(__cvta_generic_to_global(word)), "r"(bit), "r"(seen) : "memory");
-    }
-    return old;
-}
-
 template <int THREADS, int RW, bool SMEM>
 __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THREADS) k_lattice(WaveParams p) {
     extern __shared__ __align__(16) u32 s_dyn[];
     __shared__ u32 s_qn[3], s_ds[3];     // per level, rotating: queue length; its vertices' degree sum
     __shared__ long long s_cut[2];       // per level parity: the f~ that stops the source
-    __shared__ u32 s_base, s_stop, s_ovf, s_lo, s_hi;
+    __shared__ u32 s_base, s_stop, s_ovf, s_skip, s_lo, s_hi;
     __shared__ unsigned long long s_st[ST_COUNT];   // ctl's counters
     __shared__ ThrCache s_thr;                      // ctl's last snapshot of the threshold
     const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -176,6 +157,7 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
                 if (cuts) lim = cut_limit(s_thr, x, v);
             }
             s_cut[0] = lim;
+            s_skip = cuts && p.lat_lb && (long long)p.lat_lb[v] >= lim;   // its landmark bound stops it
             bm[v >> 5] = 1u << (v & 31);   // the bitmap is clean: no other bit of this word is set
             sq[0] = v;
             s_qn[0] = 1; s_qn[1] = 0;
@@ -187,7 +169,7 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
         u32 d = 0, nd = 1, a = 0, b = 1, c = 2;   // a, b, c: d, d+1, d+2 mod 3
         u64 f = 0;
         u32 lo = 0xffffffffu, hi = 0;             // bitmap words this thread set (global bitmap)
-        int end = deg == 0 ? 1 : 0;               // 1 complete, 2 cut, 3 deferred
+        int end = deg == 0 ? 1 : s_skip ? 2 : 0;   // 1 complete, 2 cut, 3 deferred
         if (ctl && deg == 0 && p.trace_lanes) lane_level(p, v, 0, 0, 1, 0);
         while (!end) {
             const u32 cnt = s_qn[a], dg = s_ds[a];
@@ -223,11 +205,7 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
                 for (int j = 0; j < RW; ++j) r[j] = v;   // no entry: a visited vertex
                 if (e < cnt) {
                     const u32 u = (e < kLatQueue ? qc[e] : __ldcg(&gqc[e])) & kLatIdMask;
-#pragma unroll
-                    for (int j = 0; j < RW; j += 4) {
-                        const uint4 t = __ldg(&rows[(size_t)u * (RW / 4) + j / 4]);
-                        r[j] = t.x; r[j + 1] = t.y; r[j + 2] = t.z; r[j + 3] = t.w;
-                    }
+                    load_row<RW>(rows, u, r);
                 }
                 u32 w[RW];
 #pragma unroll
@@ -246,15 +224,8 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
                     dsum += (r[j] >> 28) * w[j];
                     if (!SMEM && w[j]) { lo = min(lo, i); hi = max(hi, i); }
                 }
-                // places in the next queue: a scan of the warp's counts, bit by bit
-                const u32 lt = lanemask_lt();
-                u32 off = 0, total = 0;
-#pragma unroll
-                for (int k = 0; (1 << k) <= RW; ++k) {
-                    const u32 m = __ballot_sync(0xffffffffu, (found >> k) & 1u);
-                    off += __popc(m & lt) << k;
-                    total += __popc(m) << k;
-                }
+                u32 off, total;
+                warp_places<RW>(found, off, total);
                 if (total) {
                     u32 at = 0;
                     if (lane == 0) at = atomicAdd(&s_qn[b], total);

@@ -79,3 +79,59 @@ def test_bitmap_in_global_memory(B, gen, orc):
         ids, far, reach, st = h.topk(10)
     assert np.array_equal(ids, ei) and np.array_equal(far, ef) and np.array_equal(reach, er)
     assert st["sparse"] == big.n
+
+
+def _two_parts(gen, a, b, name):
+    src = np.concatenate([np.repeat(np.arange(a.n), a.degrees()), a.n + np.repeat(np.arange(b.n), b.degrees())])
+    dst = np.concatenate([a.col.astype(np.int64), a.n + b.col.astype(np.int64)])
+    return gen.csr_from_arcs(a.n + b.n, src, dst, directed=False, name=name)
+
+
+@pytest.mark.parametrize("k", [1, 10, 300])
+def test_landmark_bounds(B, gen, orc, k):
+    """From 8192 vertices on, sources are stopped by landmark bounds before their search: grids in order and
+    relabelled (interior first landmark), components without a landmark, distances that concentrate (the joint
+    bound is not taken), rows of 8, and the same without the bounds."""
+    graphs = [gen.grid_lcc(100, 95, 0.05, seed=6), gen.relabel(gen.grid_lcc(91, 99, 0.1, seed=7), seed=2),
+              _two_parts(gen, gen.grid_lcc(88, 95, 0.02, seed=8), gen.grid_lcc(90, 92, 0.02, seed=9), "two grids"),
+              _matchings(gen, 9001, 3, 4), _matchings(gen, 8200, 7, 5), gen.cycle(8192), gen.grid(9000, 1)]
+    for g in graphs:
+        ei, ef, er, _ = orc.bcm(g, k)
+        with B.BcmGraph.from_graph(g) as h:
+            for flags in (0, B.BCM_NO_PREFILTER):
+                ids, far, reach, st = h.topk(k, flags=flags)
+                assert np.array_equal(ids, ei) and np.array_equal(far, ef) and np.array_equal(reach, er), (g.name, flags)
+                assert st["sparse"] == g.n and st["completed"] + st["cut"] == g.n, (g.name, st)
+            parts = [h.topk(k, shard_index=i, shard_count=2)[:3] for i in range(2)]
+        ids, far, reach = B.bcm_topk_merge(*[np.concatenate([q[j] for q in parts]) for j in range(3)], k)
+        assert np.array_equal(ids, ei) and np.array_equal(far, ef) and np.array_equal(reach, er), (g.name, "shards")
+
+
+def test_landmark_distances_too_large(B, gen):
+    """A path longer than the bounds' distance limit (65,535): the middle vertices, from the closed form."""
+    n = 70001
+    with B.BcmGraph.from_graph(gen.path(n)) as h:
+        ids, far, reach, _ = h.topk(3)
+    m = n // 2
+    assert ids.tolist() == [m, m - 1, m + 1] and (reach == n).all()
+    assert far.tolist() == [m * (m + 1), m * (m + 1) + 1, m * (m + 1) + 1]
+
+
+def test_landmark_bounds_in_a_batch(B, gen, orc):
+    """Recorded runs (a lattice of this size still fits a batch) give the same answer on every replay."""
+    import torch
+    graphs = [gen.grid_lcc(96, 92, 0.05, seed=11), gen.grid_lcc(99, 90, 0.1, seed=12)]
+    hs = [B.BcmGraph.from_graph(g) for g in graphs]
+    out = [[torch.zeros(10, dtype=t, device="cuda") for t in (torch.int32, torch.int64, torch.int32)] for _ in graphs]
+    batch = B.BcmBatch([h.h for h in hs], [10, 10], out, torch.cuda.Stream())
+    for _ in range(2):
+        for o in out:
+            for t in o:
+                t.zero_()
+        torch.cuda.synchronize()
+        batch.run()
+        for g, o in zip(graphs, out):
+            ei, ef, er, _ = orc.bcm(g, 10)
+            assert np.array_equal(o[0].cpu().numpy(), ei) and np.array_equal(o[1].cpu().numpy(), ef)
+            assert np.array_equal(o[2].cpu().numpy(), er)
+    batch.close()
