@@ -75,8 +75,8 @@ typedef enum {
                                    Section 2.3, without its biggest-SCC refinement (results are the same) */
 #define BCM_TRACE         0x100u /* record the run's trace (read it with bcm_trace) */
 #define BCM_NO_DEFER      0x200u /* per-CTA waves never hand their sources to the grid-wide pass */
-#define BCM_NO_PREFILTER  0x400u /* no level-0/1 prefilter before the per-CTA waves (it runs on simple
-                                    graphs -- sorted rows, no repeated arc, no self-loop -- after the
+#define BCM_NO_PREFILTER  0x400u /* no prefilter (levels 0 and 1 and the walk bounds, on simple graphs --
+                                    sorted rows, no repeated arc, no self-loop -- after the first
                                     grid-wide waves; results are the same); no landmark bounds before
                                     the searches of large undirected graphs of largest degree <= 8 */
 #define BCM_NO_CUT        0x800u /* bcm_topk: no source is ever stopped by the bound, every BFS runs to its
@@ -144,7 +144,8 @@ typedef struct {
                                  entries (a power of two >= 1024; 0 = default, n/8 rounded up to a
                                  power of two within [65536, 2^21]), and a wave
                                  that makes more than half as many entries is deferred like a wide
-                                 one; otherwise (or with a value >= n) it is dense, n entries.
+                                 one (with a value given here below n, the prefilter keeps to levels
+                                 0 and 1, so that the per-CTA waves have sources); otherwise (or with a value >= n) it is dense, n entries.
                                  Results are the same either way */
 } bcm_options;
 
@@ -165,7 +166,7 @@ typedef struct {
     double   kernel_ms;       /* device time of the BFS kernels (CUDA events) */
     double   preprocess_ms;   /* device time of preprocessing done by this call */
     double   total_ms;        /* wall time of the call */
-    double   seed_ms;         /* device time of the grid-wide waves (or of the plain launches) */
+    double   seed_ms;         /* device time of the grid-wide waves and the prefilter (or of the plain launches) */
     double   wave_ms;         /* device time of the per-CTA wave kernel (or of the one-source kernel) */
     uint64_t wave_bytes;      /* algorithmic bytes the per-CTA wave kernel moved: 20 per source
                                  started, 28 per frontier word, 12 per (arc, frontier word), 32 per

@@ -286,8 +286,14 @@ struct Aux {
     uint32_t trace_n;
     uint32_t defer_n;     // sources handed back by per-CTA waves
     uint32_t head2;       // queue head of the grid-wide pass over them
-    uint32_t surv_n;      // sources the prefilter could not stop
-    uint32_t head3;       // queue head of the per-CTA waves over them
+    uint32_t walk_left[2];   // sources left by the prefilter, and by the second one
+    uint32_t walk_heavy_n[kWalkLevels + 1];
+    uint32_t walk_want;
+    uint32_t head3;       // queue head of the waves over the sources left
+    uint32_t head4;       // queue head of the per-CTA waves after the second prefilter
+    uint32_t wave_src[256];   // the grid-wide kernel's next wave
+    uint32_t wave_n;
+    uint32_t light;       // a narrow grid-wide wave has ended the grid phase
 };
 
 // Host side of a run in flight: pinned memory the run's counters are copied
@@ -324,6 +330,7 @@ struct bcm_graph {
     uint32_t* d_order = nullptr;
     uint32_t* d_xlo = nullptr;
     uint32_t* d_xhi = nullptr;
+    uint32_t* d_walk = nullptr;    // [2][n] degrees, and walks of two arcs that do not turn back (the prefilter's)
     uint32_t* d_comp = nullptr;    // component / SCC label, smallest-member order
     uint32_t* d_rrp = nullptr;     // directed: in-arcs CSR
     uint32_t* d_rcol = nullptr;
@@ -360,7 +367,7 @@ struct bcm_graph {
     cudaStream_t aux = nullptr;
     uint32_t* d_defer = nullptr;   // [n] sources deferred by per-CTA waves
     uint32_t* d_shard = nullptr;   // [n] this shard's sources, in degree order
-    uint32_t* d_surv = nullptr;    // [n] sources left for the per-CTA waves by the prefilter
+    uint32_t* d_surv = nullptr;    // the prefilter's counts and lists of sources left (carve_walks)
     HostBlock* h = nullptr;        // pinned
     unsigned long long* d_trace = nullptr;   // kTraceCap records of 4 words
     uint32_t trace_n = 0;          // records of the last finished traced run
@@ -389,6 +396,7 @@ struct Cfg {
     bool sparse;                       // per-CTA phase: one source per CTA (k_sparse)
     uint32_t sparse_qcap;
     int lat;                           // ... by k_lattice, rows of this many entries (0: k_sparse)
+    bool walks_off;                    // an explicit hashed vertex table: sources are prefiltered at levels 0 and 1 only
     bool landmarks;                    // ... with landmark bounds before the searches (top-k runs)
 };
 
@@ -483,6 +491,8 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
     // table), else dense
     if (o.cta_table && o.cta_table < g->n && (o.cta_table < 1024 || (o.cta_table & (o.cta_table - 1))))
         return fail(BCM_ERR_UNSUPPORTED, "cta_table must be a power of two >= 1024, or >= n (got %u)", o.cta_table);
+    // (a run that sizes the per-CTA phase's tables keeps that phase's sources)
+    c->walks_off = o.cta_table && o.cta_table < g->n;
     const uint32_t tab = o.cta_table ? o.cta_table : default_cta_table(g->n);
     const bool can_defer = !(c->flags & (BCM_CTA_ONLY | BCM_GRID_ONLY)) && c->defer_words &&
                            (uint64_t)g->n * c->W >= c->defer_words;
@@ -586,10 +596,11 @@ bcm_status preprocess(bcm_graph* g, double* ms) {
         if (sc > scratch) scratch = sc;
     }
     if (!g->d_order) {
-        CU(buf_get_t(&g->d_order, nb * 4), "preprocess allocation");
+        CU(buf_get_t(&g->d_order, nb * 6), "preprocess allocation");
         g->d_xlo = (uint32_t*)((char*)g->d_order + nb);
         g->d_xhi = (uint32_t*)((char*)g->d_order + 2 * nb);
         g->d_comp = (uint32_t*)((char*)g->d_order + 3 * nb);
+        g->d_walk = (uint32_t*)((char*)g->d_order + 4 * nb);
     }
     char* d_scr = nullptr;
     CU(buf_get_t(&d_scr, scratch), "preprocess scratch");
@@ -600,7 +611,7 @@ bcm_status preprocess(bcm_graph* g, double* ms) {
     const size_t dos = (degree_order_scratch_bytes(n) + 255) & ~(size_t)255;
     const size_t scs = simple_check_scratch_bytes(g->m);
     char* d_scr2 = nullptr;
-    if (buf_get_t(&d_scr2, dos + scs + 256) != cudaSuccess) {
+    if (buf_get_t(&d_scr2, dos + scs + 256 + nb) != cudaSuccess) {
         buf_put(d_scr);
         return fail(BCM_ERR_OOM, "preprocess scratch");
     }
@@ -623,11 +634,27 @@ bcm_status preprocess(bcm_graph* g, double* ms) {
             st = fail(BCM_ERR_CUDA, "degree order: %s", cudaGetErrorString(cudaGetLastError()));
             break;
         }
+        // the prefilter's counts: beside the components on the helper stream,
+        // but after them where those take fewer launches than the degree order
+        Walks K{};
+        K.c[1] = g->d_walk;
+        K.c[2] = (uint32_t*)((char*)g->d_walk + nb);
+        K.heavy_n = (uint32_t*)(d_simple + 16);
+        K.heavy = (uint32_t*)(d_scr2 + dos + scs + 256);
+        const bool walks_after = !g->directed && n <= 65536;
+        if (!walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, !g->directed, g->aux)) {
+            st = fail(BCM_ERR_CUDA, "walk counts: %s", cudaGetErrorString(cudaGetLastError()));
+            break;
+        }
         if (!g->directed) {
             uint32_t* parent = g->d_comp;
             uint32_t* size = (uint32_t*)d_scr;
             if (launch_cc_reach(g->d_rp, g->d_col, n, parent, size, g->d_xlo, g->d_xhi, d_err, s)) {
                 st = fail(BCM_ERR_CUDA, "component kernels: %s", cudaGetErrorString(cudaGetLastError()));
+                break;
+            }
+            if (walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, true, s)) {
+                st = fail(BCM_ERR_CUDA, "walk counts: %s", cudaGetErrorString(cudaGetLastError()));
                 break;
             }
             // d_comp now holds each vertex's component root (its smallest
@@ -732,6 +759,9 @@ WaveParams base_params(bcm_graph* g, const Cfg& c) {
     p.topk.thr = &a->thr;
     p.topk.ext = &a->ext;
     p.snap = &a->snap;
+    p.wave_src = a->wave_src;
+    p.wave_n = &a->wave_n;
+    p.undirected = g->directed ? 0u : 1u;
     p.slot_base = (char*)g->slots.ptr;
     p.slot_stride = cta_slot_stride(g, c);
     p.sparse_qcap = c.sparse_qcap;
@@ -861,6 +891,27 @@ bcm_status ensure_run_state(bcm_graph* g, bool trace) {
     return BCM_OK;
 }
 
+// The prefilter's memory: counts from c[3] on, the heavy list and two source lists of n entries, n bits.
+size_t walks_bytes(uint32_t n) { return (kWalkLevels + 1) * al256((size_t)n * 4) + al256((size_t)n / 8 + 4); }
+Walks carve_walks(bcm_graph* g) {
+    const size_t w = al256((size_t)g->n * 4);
+    char* p = (char*)g->d_surv;
+    auto take = [&] { char* r = p; p += w; return (uint32_t*)r; };
+    Walks K;
+    K.c[0] = nullptr;
+    K.c[1] = g->d_walk;
+    K.c[2] = (uint32_t*)((char*)g->d_walk + w);
+    for (int j = 3; j <= kWalkLevels; ++j) K.c[j] = take();
+    K.heavy = take();
+    K.list[0] = take();
+    K.list[1] = take();
+    K.keep = (uint32_t*)p;
+    K.heavy_n = g->d_aux->walk_heavy_n;
+    K.want = &g->d_aux->walk_want;
+    K.off = 0;
+    return K;
+}
+
 // Enqueues one run of the wave kernels on the graph's stream and the copies
 // of its results and counters, and returns without waiting.  exhaustive:
 // every source, no cut, outputs o_far/o_reach (n entries); else top-k with
@@ -956,15 +1007,24 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
             p.defer_n = &g->d_aux->defer_n;
             p.defer_src = g->d_defer;
         }
+        // on a simple graph, sources are tested at levels 0 to 2 from counts of
+        // walks alone as soon as a threshold exists -- after the first grid
+        // waves, or the seed wave -- and only the others are searched
+        const bool filter = g->simple && !exhaustive && !c.sparse &&
+                            !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY));
         if (grid) {
-            p.max_grid_waves = 0xffffffffu;
+            // as many waves as give k entries come before the prefilter
+            const uint32_t lanes = 64u * (uint32_t)c.grid_W;
+            p.max_grid_waves = filter ? (k + lanes - 1) / lanes : 0xffffffffu;
+            p.light = filter ? &g->d_aux->light : nullptr;
+            p.walk_want = filter ? &g->d_aux->walk_want : nullptr;
+            p.walks.off = c.walks_off ? 1u : 0u;
             p.heavy_words = (exhaustive || (c.flags & BCM_GRID_ONLY)) ? 0 : c.heavy_words;
             // default measured per level on the Chung-Lu and R-MAT workloads:
             // pull wins once the frontier's out-arcs reach about n*W/32
             p.pull_div = (c.flags & BCM_NO_PULL) ? 0u : (c.pull_div ? c.pull_div : 32u);
             rc = launch_grid_waves(p, c.grid_W, c.grid_blocks, 512, s);
         }
-        p.stats = g->d_aux->stats;
         // a graph too small for grid-wide waves: one CTA first runs the
         // first wave alone (the highest-degree sources), so the threshold
         // exists before the other waves start (otherwise they all start at
@@ -974,26 +1034,43 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         if (seed) {
             WaveParams ps = p;
             ps.max_cta_waves = 1;
+            ps.stats = g->d_aux->stats;
             rc = launch_cta_waves(ps, c.W, 1, c.threads, s);
         }
-        cudaEventRecord(g->ev[1], s);
         WaveParams pc = p;
-        // on a simple graph, the sources the grid (or the seed wave) left are
-        // first tested at levels 0 and 1 from degrees alone; the waves take
-        // the rest
-        const bool prefilter = (grid || seed) && rc == 0 && g->simple &&
-                               !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT));
-        if (prefilter) {
+        if (filter && (grid || seed) && rc == 0) {
             if (!g->d_surv) {
-                cudaError_t e = buf_get_t(&g->d_surv, (size_t)g->n * sizeof(uint32_t));
-                if (e != cudaSuccess) { cudaStreamSynchronize(s); return cuda_fail(e, "prefilter list allocation"); }
+                cudaError_t e = buf_get_t(&g->d_surv, walks_bytes(g->n));
+                if (e != cudaSuccess) { cudaStreamSynchronize(s); return cuda_fail(e, "prefilter allocation"); }
             }
-            rc = launch_prefilter(p, g->d_surv, &g->d_aux->surv_n, s);
-            pc.sources = g->d_surv;
+            Walks K = carve_walks(g);
+            K.off = c.walks_off ? 1u : 0u;
+            uint32_t* const left_n = g->d_aux->walk_left;
+            WaveParams pf = p;
+            pf.stats = g->d_aux->stats;
+            rc = launch_prefilter(pf, K, !g->directed, K.list[0], left_n, s);
+            pc.sources = K.list[0];
             pc.head = &g->d_aux->head3;
             pc.n_end = 0;
-            pc.n_end_dev = &g->d_aux->surv_n;
+            pc.n_end_dev = left_n;
+            if (grid && rc == 0) {
+                // the sources left, on the grid while their waves are wide;
+                // then those left once more against the threshold by now
+                pc.max_grid_waves = 0xffffffffu;
+                pc.pick = c.flags & BCM_TRACE_LANES ? 0u : 1u;
+                pc.walks = K;
+                pc.walk_want = nullptr;
+                rc = launch_grid_waves(pc, c.grid_W, c.grid_blocks, 512, s);
+                pf = pc;
+                pf.stats = g->d_aux->stats;
+                if (rc == 0) rc = launch_refilter(pf, K, !g->directed, K.list[1], left_n + 1, s);
+                pc.sources = K.list[1];
+                pc.head = &g->d_aux->head4;
+                pc.n_end_dev = left_n + 1;
+            }
         }
+        pc.stats = g->d_aux->stats;
+        cudaEventRecord(g->ev[1], s);
         if (rc == 0 && c.landmarks && !exhaustive) {
             // sources by landmark bound; the most central ones first, which
             // sets the threshold; the others if no bound stops them
@@ -1030,6 +1107,8 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
             q.n_end_dev = &g->d_aux->defer_n;
             q.max_grid_waves = 0xffffffffu;
             q.heavy_words = 0;
+            q.light = nullptr;
+            q.walk_want = nullptr;
             q.defer_words = 0;
             q.pull_div = (c.flags & BCM_NO_PULL) ? 0u : (c.pull_div ? c.pull_div : 32u);
             q.stats = g->d_aux->seed_stats;
@@ -1707,7 +1786,7 @@ uint64_t bcm_workspace_bytes(bcm_graph_t g, const bcm_options* opt) {
     if (!g->preprocessed && preprocess(g, nullptr) != BCM_OK) return 0;   // the default kernels depend on it
     Cfg c;
     if (resolve(g, opt, &c)) return 0;
-    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * (12 + 4 * c.lat) +
+    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * (8 + 4 * c.lat) + walks_bytes(g->n) +
            (c.landmarks ? landmark_bytes(g->n) : 0);
 }
 

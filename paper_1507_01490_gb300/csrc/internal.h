@@ -74,6 +74,18 @@ struct HeavyEntry {
     uint32_t g, pad;        // word group
 };
 
+// The prefilter's working memory (n entries an array; keep: n bits).
+constexpr int kWalkLevels = 4;
+struct Walks {
+    uint32_t* c[kWalkLevels + 1];   // c[j][v]: walks of j arcs from v that never turn straight back (j >= 1)
+    uint32_t* heavy;                // rows summed by whole blocks
+    uint32_t* list[2];              // sources left, round by round
+    uint32_t* keep;                 // which positions of the source list stay
+    uint32_t* heavy_n;              // [kWalkLevels + 1]
+    uint32_t* want;                 // the last c[j] there is (at least 2)
+    uint32_t off;                   // no more than c[2]
+};
+
 struct WaveParams {
     GraphDev g;
     uint32_t footnote;       // undirected: gamma~ uses deg(u)-1 for d >= 1
@@ -134,6 +146,14 @@ struct WaveParams {
     uint32_t* trace_n;       // records written (may exceed trace_cap; the excess is dropped)
     uint32_t trace_lanes;    // also record every lane's level state and end (needs trace)
     uint32_t nocut;          // top-k runs: never stop a source (every BFS runs to its end)
+    // grid-wide kernel: the next wave's sources, picked by the leader block -- the next of the
+    // queue, or (pick) the next that the walk bounds do not stop
+    uint32_t* wave_src;      // [256]
+    uint32_t* wave_n;
+    uint32_t pick, undirected;
+    uint32_t* walk_want;     // receives, when the launch ends, how many walk counts the prefilter wants
+    Walks walks;
+    uint32_t* light;         // grid-wide kernel: set when a narrow wave ended it; set on entry: nothing to do
     Threshold* snap;         // grid-wide and plain kernels: the threshold all blocks cut with (see store_snapshot)
 };
 
@@ -181,9 +201,16 @@ int launch_scc_bounds(const uint32_t* rp, const uint32_t* col, const uint32_t* r
 // ---- msbfs.cu
 int launch_grid_waves(const WaveParams& p, int W, int blocks, int threads, cudaStream_t s);
 int launch_cta_waves(const WaveParams& p, int W, int blocks, int threads, cudaStream_t s);
-// level-0/1 stopping rule for sources p.sources[*p.head .. p.n_end) of a simple graph;
-// the sources it cannot stop are appended to out (count in *out_n)
-int launch_prefilter(const WaveParams& p, uint32_t* out, uint32_t* out_n, cudaStream_t s);
+// c[1] and c[2] (K.heavy: n entries of scratch, K.heavy_n: kWalkLevels + 1)
+int launch_walk_base(const uint32_t* rp, const uint32_t* col, uint32_t n, const Walks& K, bool undirected,
+                     cudaStream_t s);
+// Stopping rule at levels 0 and 1 and walk bounds for the sources p.sources[*p.head .. end) of a simple
+// graph; those it cannot stop go to out in the same order, their count to *out_n (device memory).
+int launch_prefilter(const WaveParams& p, const Walks& K, bool undirected, uint32_t* out, uint32_t* out_n,
+                     cudaStream_t s);
+// the same for p's sources with the counts already there, against the threshold by now
+int launch_refilter(const WaveParams& p, const Walks& K, bool undirected, uint32_t* out, uint32_t* out_n,
+                    cudaStream_t s);
 int launch_plain_source(const WaveParams& p, uint32_t it, uint32_t* stamp, uint32_t* lists,
                         int blocks, int threads, cudaStream_t s);
 

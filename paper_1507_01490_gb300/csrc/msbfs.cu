@@ -1012,113 +1012,399 @@ __device__ __noinline__ void flush_completions(const WaveParams& p, const u32* c
 // v's BFS is known without expanding it: Gamma_1 = N(v), so gamma_1 = deg(v),
 // n_1 = 1 + deg(v), f_1 = deg(v), and gamma~_2 (Table 1, with the footnote's
 // deg(u) - 1 on undirected graphs) = sum over u in N(v) of deg(u) - footnote.
-// One warp per source applies the stopping rule at levels 0 and 1, exactly as
-// a wave would, against the threshold the grid-wide waves left (no higher
-// than the one a later wave would read); the sources it cannot stop go to
-// `out` for the per-CTA waves.  Sources p.sources[*p.head .. p.n_end).
-__global__ void __launch_bounds__(256) k_prefilter(WaveParams p, u32* out, u32* out_n) {
+// Further levels follow from counts of walks that never turn straight back:
+// with c_1 = deg, c_2 = gamma~_2 and
+//     c_{j+1}(v) = sum over u in N(v) of c_j(u) - (deg(v) - 1) c_{j-1}(v)
+// (the walks that go to u and straight back left out; on digraphs the plain
+// sum), gamma_j <= c_j, and every vertex of R(v) beyond level J is at distance
+// J + 1 or more, so for each J
+//     f(v) >= sum_{j <= J} j c_j + (J + 1) (r(v) - 1 - sum_{j <= J} c_j),
+// Lemma 1's form at d = J - 1 with upper counts in place of the exact ones.
+// One sum over all rows per level thus does for every source at once what a
+// search per source would have to do.  On Barabasi-Albert graphs (m = 4) the
+// first tests leave every source and J = 3 about a hundred; at m = 2, J = 4
+// leaves 3%.  Kernel time, k_prefilter with levels 0 and 1 only -> now: BA
+// 2^20, m = 4, top-10, 43.1 (16,381 per-CTA waves) -> 1.43 ms; BA 10^6, m = 2,
+// top-10, 1,917 -> 19 ms, m = 8, top-100, 919 -> 9.9 ms; Chung-Lu 2^20, top-10,
+// 1.47 -> 1.21 ms (the tests come after the first wave instead of the fifth).
+//
+// The bound at J tends to J + 1 per vertex reached, so it can only stop
+// sources while the k-th entry's mean distance F / (r - 1) is below that: c_3
+// is summed where that distance is above 2.75, c_4 above 3.75 (Chung-Lu and
+// R-MAT, 2.1 to 2.6, pay for neither).
+//
+//   k_walk_degree, k_walk_sum, k_walk_heavy   c_1; c_{j+1} from c_j.  c_1 and
+//                 c_2 belong to the graph's preprocessing
+//   k_prefilter   32 consecutive positions of the source list per warp: the
+//                 stopping rule at levels 0 and 1 as a wave would apply it, then
+//                 the bounds; one bit per position says that it stays
+//   k_compact     the sources that stay, in the list's order (by degree)
+//   k_filter_small   all of it from c_3 on in one launch, by one cluster of
+//                 eight CTAs, on graphs of at most 65,536 vertices (six launches
+//                 of 3 us each otherwise)
+constexpr u32 kWalkHeavy = 1024;         // longer rows are summed by a whole block
+constexpr u32 kWalkMany = 1u << 31;      // a count that is this large or larger (n < 2^30)
+constexpr u32 kWalkSmall = 65536;        // graphs for k_filter_small
+
+// The last c_j wanted, given the k-th key.
+__device__ __forceinline__ u32 walk_levels(const WaveParams& p, const Walks& K) {
+    ThrCache t;
+    t.valid = 0; t.N = 0; t.F = 1; t.id = 0;
+    read_thresholds(p.topk, t);
+    if (K.off || p.trace_lanes || !t.valid || t.N == 0) return 2;
+    const double mean = (double)t.F / sqrt((double)t.N);
+    return mean > 3.75 ? 4u : mean > 2.75 ? 3u : 2u;
+}
+
+__global__ void k_walk_degree(GraphDev G, u32* deg, u32* heavy_n) {
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    if (blockIdx.x == 0 && threadIdx.x <= kWalkLevels) heavy_n[threadIdx.x] = 0;
+    for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < G.n; v += stride)
+        deg[v] = __ldg(&G.rp[v + 1]) - __ldg(&G.rp[v]);
+}
+
+// A row's sum made a count: walks straight back left out, large ones held.
+__device__ __forceinline__ u32 walk_count(const Walks& K, int j, u32 v, u32 deg, u64 sum, bool many, bool undirected) {
+    if (undirected) {
+        const u64 back = j == 2 ? deg : (u64)(deg - 1) * K.c[j - 2][v];
+        sum = sum > back ? sum - back : 0;
+    }
+    return many || sum >= kWalkMany ? kWalkMany : (u32)sum;
+}
+
+// c_j from c_{j-1}: one thread per vertex; rows over 32 by the warp, over
+// kWalkHeavy listed for walk_heavy.
+// (LAST: the counts were written by an earlier launch, so they may be cached in L1)
+template <bool LAST>
+__device__ __forceinline__ u32 walk_load(const u32* p) { return LAST ? __ldg(p) : __ldcg(p); }
+
+template <bool LAST>
+__device__ __forceinline__ void walk_sums(const GraphDev& G, const Walks& K, int j, bool undirected, size_t tid,
+                                          size_t stride) {
+    const u32* in = K.c[j - 1];
+    const u32 lane = threadIdx.x & 31;
+    for (size_t v0 = tid - lane; v0 < G.n; v0 += stride) {
+        const size_t v = v0 + lane;
+        u32 b = 0, deg = 0;
+        u64 sum = 0;
+        bool many = false;
+        if (v < G.n) {
+            b = __ldg(&G.rp[v]);
+            deg = __ldg(&G.rp[v + 1]) - b;
+        }
+        const bool heavy = deg > kWalkHeavy;
+        const bool wide = deg > 32 && !heavy;
+        if (!wide && !heavy) {
+            for (u32 i = 0; i < deg; i += 4) {   // four neighbours' counts in flight
+                u32 u[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) u[q] = i + q < deg ? __ldg(&G.col[b + i + q]) : 0xffffffffu;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (u[q] != 0xffffffffu) {
+                        const u32 t = walk_load<LAST>(&in[u[q]]);
+                        many = many || t == kWalkMany;
+                        sum += t;
+                    }
+            }
+        }
+        u32 todo = __ballot_sync(0xffffffffu, wide);
+        while (todo) {
+            const int l0 = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const u32 cb = __shfl_sync(0xffffffffu, b, l0), cd = __shfl_sync(0xffffffffu, deg, l0);
+            u64 part = 0;
+            bool m = false;
+            for (u32 i = lane; i < cd; i += 128) {
+                u32 u[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) u[q] = i + 32 * q < cd ? __ldg(&G.col[cb + i + 32 * q]) : 0xffffffffu;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (u[q] != 0xffffffffu) {
+                        const u32 t = walk_load<LAST>(&in[u[q]]);
+                        m = m || t == kWalkMany;
+                        part += t;
+                    }
+            }
+            for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+            m = __any_sync(0xffffffffu, m);
+            if (lane == (u32)l0) { sum = part; many = m; }
+        }
+        warp_append(heavy, (u32)v, K.heavy, K.heavy_n + j);
+        if (v < G.n && !heavy) K.c[j][v] = walk_count(K, j, (u32)v, deg, sum, many, undirected);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_walk_sum(GraphDev G, Walks K, int j, bool undirected) {
+    if (j > 2 && (u32)j > *K.want) return;
+    walk_sums<true>(G, K, j, undirected, blockIdx.x * (size_t)blockDim.x + threadIdx.x, (size_t)gridDim.x * blockDim.x);
+}
+
+// The listed rows, one block each, eight counts in flight per thread.
+template <bool LAST>
+__device__ __forceinline__ void walk_heavy(const GraphDev& G, const Walks& K, int j, bool undirected) {
+    __shared__ unsigned long long s_sum;
+    __shared__ u32 s_many;
+    const u32* in = K.c[j - 1];
+    const u32 hn = __ldcg(&K.heavy_n[j]), T = blockDim.x;
+    for (u32 h = blockIdx.x; h < hn; h += gridDim.x) {
+        if (threadIdx.x == 0) { s_sum = 0; s_many = 0; }
+        __syncthreads();
+        const u32 v = __ldcg(&K.heavy[h]), b = __ldg(&G.rp[v]), e = __ldg(&G.rp[v + 1]);
+        u64 part = 0;
+        bool m = false;
+        for (u64 i = b + threadIdx.x; i < e; i += T * 8) {
+            u32 u[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) u[q] = i + T * q < e ? __ldg(&G.col[i + T * q]) : 0xffffffffu;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (u[q] != 0xffffffffu) {
+                    const u32 t = walk_load<LAST>(&in[u[q]]);
+                    m = m || t == kWalkMany;
+                    part += t;
+                }
+        }
+        for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, (unsigned long long)part);
+        if (m) s_many = 1;
+        __syncthreads();
+        if (threadIdx.x == 0) K.c[j][v] = walk_count(K, j, v, e - b, s_sum, s_many != 0, undirected);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(512) k_walk_heavy(GraphDev G, Walks K, int j, bool undirected) {
+    if (j > 2 && (u32)j > *K.want) return;
+    walk_heavy<true>(G, K, j, undirected);
+}
+
+// Does one of the bounds with J = 2 .. last stop v?  Each J is a line in x =
+// r(v), so the two ends of its range decide (Lemma 2's argument).
+__device__ __forceinline__ bool walk_stops(const Walks& K, int last, u32 v, u32 xlo, u32 xhi, const ThrCache& t) {
+    const __int128 N = t.N, rl = (__int128)t.F * ((__int128)xlo - 1) * ((__int128)xlo - 1),
+                   rh = (__int128)t.F * ((__int128)xhi - 1) * ((__int128)xhi - 1);
+    long long sum = 0, far = 0;   // of c_j and j c_j
+    for (int j = 1; j <= last; ++j) {
+        const u32 c = K.c[j][v];
+        if (c == kWalkMany) return false;   // no line further on is better
+        sum += c;
+        far += (long long)j * c;
+        if (j < 2) continue;
+        const __int128 l = (__int128)(far + (j + 1) * ((long long)xlo - 1 - sum)) * N;
+        const __int128 h = (__int128)(far + (j + 1) * ((long long)xhi - 1 - sum)) * N;
+        if ((l > rl && h > rh) || (l >= rl && h >= rh && v > t.id)) return true;
+    }
+    return false;
+}
+
+// Sources p.sources[begin .. n_end): bit `position` of K.keep says that it
+// stays.  `use`: the last count there.
+__device__ __forceinline__ void filter_sources(const WaveParams& p, const Walks& K, bool undirected, int use, u32 begin,
+                                               u32 n_end, const ThrCache& thr, size_t gw, size_t gnw, LocalStats& st,
+                                               BlockStats& bst) {
+    const GraphDev& G = p.g;
+    const u32 lane = threadIdx.x & 31;
+    u32 ncut = 0, ndone = 0;
+    for (size_t word = (begin >> 5) + gw; word * 32 < n_end; word += gnw) {
+        const size_t pos = word * 32 + lane;
+        const bool have = pos >= begin && pos < n_end;
+        bool stays = have;
+        if (have && thr.valid) {
+            const u32 v = __ldg(&p.sources[pos]);
+            const u32 deg = __ldcg(&K.c[1][v]), c2 = __ldcg(&K.c[2][v]), xlo = __ldg(&G.xlo[v]);
+            const u32 xhi = undirected ? xlo : __ldg(&G.xhi[v]);
+            // gamma~_2 as BFSCut has it: with the footnote or without
+            const u32 two = c2 + (undirected && !p.footnote && c2 != kWalkMany ? deg : 0u);
+            if (p.trace_lanes) lane_level(p, v, 0, 0, 1, deg);
+            if (deg == 0) {
+                // R(v) = {v}: complete with key (0, 1); it only goes on (to be
+                // merged by a wave) if it ranks before the k-th
+                if (!ranks_before(0, 1, v, thr.N, thr.F, thr.id)) {
+                    stays = false;
+                    ++ndone;
+                    if (p.trace_lanes) lane_end(p, v, 0, 0, 1, false);
+                }
+            } else if (bfscut_stops(0, deg, 0, 1, xlo, xhi, v, thr)) {
+                stays = false;
+                ++ncut;
+                if (p.trace_lanes) lane_end(p, v, 0, 0, 1, true);
+            } else {
+                if (p.trace_lanes) lane_level(p, v, 1, deg, 1 + deg, two);
+                // (no lane record of the walk bounds: they are no level of a search)
+                const bool one = bfscut_stops(deg, two, 1, 1 + deg, xlo, xhi, v, thr);
+                if (one || (use > 2 && walk_stops(K, use, v, xlo, xhi, thr))) {
+                    stays = false;
+                    ++ncut;
+                    st.mvis += deg;   // level 0 was expanded
+                    st.arcwords += deg;
+                    if (p.trace_lanes) lane_end(p, v, 1, deg, 1 + deg, true);
+                }
+            }
+        }
+        const u32 m = __ballot_sync(0xffffffffu, stays);
+        if (lane == 0) K.keep[word] = m;
+    }
+    ncut = __reduce_add_sync(0xffffffffu, ncut);
+    ndone = __reduce_add_sync(0xffffffffu, ndone);
+    if (lane == 0 && ncut) bstat_add(bst, ST_CUT, ncut);
+    if (lane == 0 && ndone) bstat_add(bst, ST_COMPLETED, ndone);
+}
+
+__global__ void __launch_bounds__(256) k_prefilter(WaveParams p, Walks K, bool undirected) {
     __shared__ ThrCache s_thr;
     __shared__ BlockStats s_bst;
-    __shared__ u32 s_begin;
-    const GraphDev& G = p.g;
+    __shared__ u32 s_begin, s_want;
     if (threadIdx.x == 0) {
         s_thr.valid = 0; s_thr.N = 0; s_thr.F = 1; s_thr.id = 0;
         read_thresholds(p.topk, s_thr);
         s_begin = vload(p.head);
+        s_want = *K.want;
     }
     bstat_init(s_bst);
     __syncthreads();
     LocalStats st;
-    const u32 lane = threadIdx.x & 31;
-    const size_t gw = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5;
-    const size_t gnw = ((size_t)gridDim.x * blockDim.x) >> 5;
-    // 32 sources per warp step, one per thread; a source with more than 32
-    // neighbours has its degree sum taken by the whole warp afterwards.  In
-    // each pass over gnw*32 positions, lane l of warp w takes position
-    // l*gnw + w: the sources come by degree, so consecutive positions would
-    // give the first warps all the hubs (and the step's critical path)
-    for (size_t base = s_begin; base < p.n_end; base += gnw * 32) {
-        const size_t pos = base + lane * gnw + gw;
-        const bool have = pos < p.n_end;
-        u32 v = 0, b = 0, deg = 0, xlo = 0, xhi = 0;
-        bool cut = false, done = !have || !s_thr.valid;
-        if (have) {
-            v = __ldg(&p.sources[pos]);
-            b = __ldg(&G.rp[v]);
-            deg = __ldg(&G.rp[v + 1]) - b;
-        }
-        if (!done && p.trace_lanes) lane_level(p, v, 0, 0, 1, deg);
-        if (!done && deg == 0) {
-            // R(v) = {v}: complete with key (0, 1); it only goes on (to be
-            // merged by a wave) if it ranks before the k-th
-            done = true;
-            if (!ranks_before(0, 1, v, s_thr.N, s_thr.F, s_thr.id)) {
-                cut = true;
-                bstat_add(s_bst, ST_COMPLETED, 1);
-                if (p.trace_lanes) lane_end(p, v, 0, 0, 1, false);
-            }
-        }
-        if (!done) {
-            xlo = __ldg(&G.xlo[v]);
-            xhi = __ldg(&G.xhi[v]);
-            if (bfscut_stops(0, deg, 0, 1, xlo, xhi, v, s_thr)) {
-                cut = done = true;
-                bstat_add(s_bst, ST_CUT, 1);
-                if (p.trace_lanes) lane_end(p, v, 0, 0, 1, true);
-            }
-        }
-        // level 1: gamma~_2 = sum over N(v) of deg(u) - footnote
-        u64 g2 = 0;
-        const bool serial = !done && deg <= 32;
-        if (serial) {   // four neighbours per step: their col entries, then their degrees, in flight together
-            for (u32 i = 0; i < deg; i += 4) {
-                u32 u[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) u[j] = i + j < deg ? __ldg(&G.col[b + i + j]) : 0xffffffffu;
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (u[j] != 0xffffffffu) g2 += __ldg(&G.rp[u[j] + 1]) - __ldg(&G.rp[u[j]]) - p.footnote;
-            }
-        }
-        u32 big = __ballot_sync(0xffffffffu, !done && !serial);
-        while (big) {
-            const int l0 = __ffs(big) - 1;
-            big &= big - 1;
-            const u32 cb = __shfl_sync(0xffffffffu, b, l0), cd = __shfl_sync(0xffffffffu, deg, l0);
-            u64 part = 0;
-            for (u32 i = lane; i < cd; i += 32) {
-                const u32 u = __ldg(&G.col[cb + i]);
-                part += __ldg(&G.rp[u + 1]) - __ldg(&G.rp[u]) - p.footnote;
-            }
-            for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-            if (lane == (u32)l0) g2 = part;
-        }
-        if (!done) {
-            if (p.trace_lanes) lane_level(p, v, 1, deg, 1 + deg, (u32)g2);
-            if (bfscut_stops(deg, g2, 1, 1 + deg, xlo, xhi, v, s_thr)) {
-                cut = true;
-                bstat_add(s_bst, ST_CUT, 1);
-                st.mvis += deg;       // level 0 was expanded
-                st.arcwords += deg;
-                if (p.trace_lanes) lane_end(p, v, 1, deg, 1 + deg, true);
-            }
-        }
-        const bool keep = have && !cut;
-        const u32 m = __ballot_sync(0xffffffffu, keep);
-        if (m) {
-            u32 at = 0;
-            if (lane == 0) at = atomicAdd(out_n, (u32)__popc(m));
-            at = __shfl_sync(0xffffffffu, at, 0);
-            if (keep) out[at + __popc(m & lanemask_lt())] = v;
-        }
-    }
+    const u32 n_end = p.n_end_dev ? vload(p.n_end_dev) : p.n_end;
+    // warps numbered across blocks first
+    filter_sources(p, K, undirected, (int)s_want, s_begin, n_end, s_thr,
+                   ((size_t)(threadIdx.x >> 5) * gridDim.x) + blockIdx.x, ((size_t)gridDim.x * blockDim.x) >> 5, st,
+                   s_bst);
     __syncthreads();
     flush_stats(st, s_bst, p.stats);
 }
 
-int launch_prefilter(const WaveParams& p, uint32_t* out, uint32_t* out_n, cudaStream_t s) {
-    k_prefilter<<<152 * 8, 256, 0, s>>>(p, out, out_n);
+// The kept sources in the list's order: block b of kCompactBlocks takes the
+// b-th share of keep's words and counts the bits before it by itself (at most
+// n / 32 words, read by 1024 threads).
+constexpr u32 kCompactBlocks = 64;
+__device__ __forceinline__ void compact_sources(const WaveParams& p, const u32* keep, u32 head, u32 n_end, u32 blk,
+                                                u32 nblk, u32* out, u32* out_n) {
+    __shared__ u32 s_before, s_warp[32];
+    const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
+    const u32 w0 = head >> 5, w1 = (n_end + 31) / 32;
+    if (w0 >= w1) {
+        if (blk == 0 && tid == 0) *out_n = 0;
+        return;
+    }
+    const u32 share = (w1 - w0 + nblk - 1) / nblk;
+    const u32 b = w0 + blk * share < w1 ? w0 + blk * share : w1, e = b + share < w1 ? b + share : w1;
+    if (tid == 0) s_before = 0;
+    __syncthreads();
+    u32 before = 0;
+    for (u32 w = w0 + tid; w < b; w += T) before += __popc(__ldcg(&keep[w]));
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0 && before) atomicAdd(&s_before, before);
+    __syncthreads();
+    u32 base = s_before;
+    for (u32 c = b; c < e; c += T) {
+        const u32 w = c + tid;
+        u32 m = w < e ? __ldcg(&keep[w]) : 0;
+        u32 incl = __popc(m);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u32 t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (u32)o) incl += t;
+        }
+        __syncthreads();
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        u32 off = base, all = 0;
+        for (u32 i = 0; i < T / 32; ++i) {
+            if (i < wid) off += s_warp[i];
+            all += s_warp[i];
+        }
+        off += incl - __popc(m);
+        for (; m; m &= m - 1) out[off++] = p.sources[(size_t)w * 32 + __ffs(m) - 1];
+        base += all;
+    }
+    if (blk == nblk - 1 && tid == 0) *out_n = base;
+}
+
+__global__ void __launch_bounds__(1024) k_compact(WaveParams p, Walks K, u32* out, u32* out_n) {
+    const u32 n_end = p.n_end_dev ? vload(p.n_end_dev) : p.n_end;
+    compact_sources(p, K.keep, vload(p.head), n_end, blockIdx.x, kCompactBlocks, out, out_n);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+constexpr int kSmallCtas = 8;
+constexpr int kSmallThreads = 1024;
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads)
+k_filter_small(WaveParams p, Walks K, bool undirected, bool sums, u32* out, u32* out_n) {
+    __shared__ ThrCache s_thr;
+    __shared__ BlockStats s_bst;
+    __shared__ u32 s_begin;
+    const size_t tid = blockIdx.x * (size_t)kSmallThreads + threadIdx.x, stride = (size_t)kSmallCtas * kSmallThreads;
+    if (threadIdx.x == 0) {
+        s_thr.valid = 0; s_thr.N = 0; s_thr.F = 1; s_thr.id = 0;
+        read_thresholds(p.topk, s_thr);
+        s_begin = vload(p.head);
+        // one CTA decides for all: a key offered meanwhile may reach only some
+        if (sums && blockIdx.x == 0) *K.want = walk_levels(p, K);
+    }
+    bstat_init(s_bst);
+    cluster_barrier();
+    const u32 want = __ldcg(K.want);
+    for (u32 j = 3; sums && j <= want; ++j) {
+        walk_sums<false>(p.g, K, (int)j, undirected, tid, stride);
+        cluster_barrier();
+        if (__ldcg(&K.heavy_n[j])) {   // (the same in every CTA)
+            walk_heavy<false>(p.g, K, (int)j, undirected);
+            cluster_barrier();
+        }
+    }
+    LocalStats st;
+    const u32 n_end = p.n_end_dev ? vload(p.n_end_dev) : p.n_end;
+    filter_sources(p, K, undirected, (int)want, s_begin, n_end, s_thr, tid >> 5, stride >> 5, st, s_bst);
+    __syncthreads();
+    flush_stats(st, s_bst, p.stats);
+    cluster_barrier();
+    if (blockIdx.x == 0) compact_sources(p, K.keep, s_begin, n_end, 0, 1, out, out_n);
+}
+
+static int launch_filter_small(const WaveParams& p, const Walks& K, bool undirected, bool sums, uint32_t* out,
+                               uint32_t* out_n, cudaStream_t s) {
+    k_filter_small<<<kSmallCtas, kSmallThreads, 0, s>>>(p, K, undirected, sums, out, out_n);
     note_launch();
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int launch_refilter(const WaveParams& p, const Walks& K, bool undirected, uint32_t* out, uint32_t* out_n,
+                    cudaStream_t s) {
+    if (p.g.n <= kWalkSmall) return launch_filter_small(p, K, undirected, false, out, out_n, s);
+    const unsigned b = (p.g.n + 255) / 256 < 152 * 4 ? (p.g.n + 255) / 256 : 152 * 4;
+    k_prefilter<<<b, 256, 0, s>>>(p, K, undirected);
+    k_compact<<<kCompactBlocks, 1024, 0, s>>>(p, K, out, out_n);
+    note_launch(2);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int launch_prefilter(const WaveParams& p, const Walks& K, bool undirected, uint32_t* out, uint32_t* out_n,
+                     cudaStream_t s) {
+    if (p.g.n <= kWalkSmall) return launch_filter_small(p, K, undirected, true, out, out_n, s);
+    const unsigned b = (p.g.n + 255) / 256 < 152 * 8 ? (p.g.n + 255) / 256 : 152 * 8;
+    for (int j = 3; j <= kWalkLevels; ++j) {
+        k_walk_sum<<<b, 256, 0, s>>>(p.g, K, j, undirected);
+        k_walk_heavy<<<152 * 4, 512, 0, s>>>(p.g, K, j, undirected);
+    }
+    note_launch(2 * (kWalkLevels - 2));
+    return launch_refilter(p, K, undirected, out, out_n, s);
+}
+
+int launch_walk_base(const uint32_t* rp, const uint32_t* col, uint32_t n, const Walks& K, bool undirected,
+                     cudaStream_t s) {
+    GraphDev G;
+    G.n = n;
+    G.rp = rp;
+    G.col = col;
+    const unsigned b = (n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8;
+    k_walk_degree<<<b, 256, 0, s>>>(G, K.c[1], K.heavy_n);
+    k_walk_sum<<<b, 256, 0, s>>>(G, K, 2, undirected);
+    k_walk_heavy<<<152 * 4, 512, 0, s>>>(G, K, 2, undirected);
+    note_launch(3);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1678,6 +1964,66 @@ __device__ __forceinline__ bool pull_wanted(const WaveParams& p, int W, u64 farc
 #define BCM_GRID_MIN_BLOCKS 2
 #endif
 
+// The next wave's sources, by the leader block (the whole of it) while the
+// others wait at the barrier: the next L of the queue, or, with p.pick, the
+// next L that neither the stopping rule at levels 0 and 1 nor the walk bounds
+// stop against the threshold by now (the prefilter ran against an earlier
+// one: on Barabasi-Albert n = 150,000, m = 3, top-100, 36,000 sources passed
+// it and 282 waves ran, 100 ms; with the picking 30 waves, 13.3 ms).
+__device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, const ThrCache& thr, BlockStats& bst,
+                                       u64* mvis) {
+    __shared__ u32 s_cnt[32], s_last;
+    const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
+    __syncthreads();
+    u32 base = vload(p.head), cnt = 0;
+    const int use = p.pick ? (int)__ldcg(p.walks.want) : 0;
+    while (cnt < L && base < n_end) {
+        const u32 pos = base + tid;
+        const bool have = pos < n_end;
+        bool keep = have, done = false;
+        u32 v = 0, deg = 0;
+        if (have) {
+            v = __ldg(&p.sources[pos]);
+            if (p.pick && thr.valid) {
+                deg = p.walks.c[1][v];
+                const u32 c2 = p.walks.c[2][v], xlo = __ldg(&p.g.xlo[v]), xhi = __ldg(&p.g.xhi[v]);
+                if (deg == 0) {
+                    keep = ranks_before(0, 1, v, thr.N, thr.F, thr.id);
+                    done = !keep;
+                } else {
+                    const u32 two = c2 + (p.undirected && !p.footnote && c2 != kWalkMany ? deg : 0u);
+                    keep = !bfscut_stops(0, deg, 0, 1, xlo, xhi, v, thr) &&
+                           !bfscut_stops(deg, two, 1, 1 + deg, xlo, xhi, v, thr) &&
+                           !(use > 2 && walk_stops(p.walks, use, v, xlo, xhi, thr));
+                }
+            }
+        }
+        const u32 m = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) s_cnt[wid] = __popc(m);
+        if (tid == 0) s_last = base + blockDim.x < n_end ? base + blockDim.x : n_end;
+        __syncthreads();
+        u32 rank = cnt + __popc(m & lanemask_lt()), total = 0;
+        for (u32 w = 0; w < nwarp; ++w) {
+            if (w < wid) rank += s_cnt[w];
+            total += s_cnt[w];
+        }
+        if (keep && rank < L) p.wave_src[rank] = v;
+        if (keep && rank == L - 1) s_last = pos + 1;   // the wave is full: the rest stays in the queue
+        __syncthreads();
+        base = s_last;
+        cnt = cnt + total < L ? cnt + total : L;
+        if (have && !keep && pos < base) {
+            bstat_add(bst, done ? ST_COMPLETED : ST_CUT, 1);
+            *mvis += deg;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        vstore(p.head, base);
+        vstore(p.wave_n, cnt);
+    }
+}
+
 template <int W, int THREADS>
 __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(WaveParams p) {
     constexpr int L = 64 * W;
@@ -1723,19 +2069,25 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
         store_snapshot(p.snap, s_thr);
     }
     bstat_init(s_bst);
+    // an earlier launch of this run met a narrow wave: the per-CTA waves take the rest
+    if (p.light && vload(p.light)) return;
+    if (leader) {
+        __syncthreads();   // s_thr, s_bst
+        pick_wave(p, L, n_end, s_thr, s_bst, &st.mvis);
+    }
     bool ok = grid_sync(p.bar, gridDim.x, p.barrier_limit_ns, p.err);
 
     for (u32 wave = 0; ok && wave < p.max_grid_waves; ++wave) {
-        if (tid == 0) s_base = vload(p.head);
+        if (tid == 0) s_base = vload(p.wave_n);
         __syncthreads();
-        const u32 base = s_base;
-        if (base >= n_end) break;
+        const u32 wave_n = s_base;
+        if (wave_n == 0) break;
         if (tid < L) {
             bool alive = false;
             s_cg[tid] = 0;
             s_cs[tid] = 0;
-            if (base + tid < n_end) {
-                u32 v = __ldg(&p.sources[base + tid]);
+            if (tid < wave_n) {
+                u32 v = vload(&p.wave_src[tid]);
                 u32 deg = __ldg(&G.rp[v + 1]) - __ldg(&G.rp[v]);
                 s_src[tid] = v; s_nd[tid] = 1; s_f[tid] = 0; s_gt[tid] = deg;
                 s_xlo[tid] = __ldg(&G.xlo[v]); s_xhi[tid] = __ldg(&G.xhi[v]);
@@ -1953,14 +2305,22 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
                 p.gchunk[0] = 0;
                 p.gchunk[1] = 0;
                 *p.glog_n = 0;
-                *p.head = base + L;
+            }
+        }
+        // light (its levels averaged fewer than heavy_words frontier words):
+        // hand the rest of the queue over to the CTAs
+        const bool light = !p.exhaustive && wave_entries < p.heavy_words * (u64)(d ? d : 1);
+        if (leader) {
+            if (light) {
+                if (tid == 0 && p.light) vstore(p.light, 1u);
+            } else if (wave + 1 < p.max_grid_waves) {
+                pick_wave(p, L, n_end, s_thr, s_bst, &st.mvis);
             }
         }
         if (!(ok = grid_sync(p.bar, gridDim.x, p.barrier_limit_ns, p.err))) break;
-        // light (its levels averaged fewer than heavy_words frontier words):
-        // hand the rest of the queue over to the CTAs
-        if (!p.exhaustive && wave_entries < p.heavy_words * (u64)(d ? d : 1)) break;
+        if (light) break;
     }
+    if (leader && tid == 0 && p.walk_want) *p.walk_want = walk_levels(p, p.walks);
     __syncthreads();
     flush_stats(st, s_bst, p.stats);
 }
