@@ -102,7 +102,12 @@ typedef enum {
  * runs skip the grid kernel).  A per-CTA wave that turns out wide after all
  * is stopped and its sources run again on the grid kernel after the
  * per-CTA phase (see defer_words).  Exhaustive runs stay on the grid
- * kernel (with BCM_SPARSE, on the one-source kernel).  Levels of grid waves
+ * kernel (with BCM_SPARSE, on the one-source kernel); with no flag but
+ * BCM_OUT_DEVICE / BCM_NO_FOOTNOTE they run on the all-pairs kernel (targets
+ * as lanes) where its bit planes stay in L2 (up to about 130,000 vertices), and
+ * top-k runs of small graphs with no launch parameter set take their answer
+ * from every vertex's farness by that kernel (n <= 16,384 and n m below 2^30,
+ * or 2^32 for k > 32 or n < 9,728).  Levels of grid waves
  * run by push (each frontier vertex
  * sets its lanes' bits in its out-neighbours) or, when the frontier's arcs
  * are a large share of the graph's, by pull (each vertex with lanes still

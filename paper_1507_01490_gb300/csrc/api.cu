@@ -58,7 +58,7 @@ static bcm_status cuda_fail(cudaError_t e, const char* what) {
 // of one layout overlap the bit arrays of another.
 struct Layout {
     uint32_t n = 0, W = 0, blocks = 0, entries = 0;   // entries: the vertex tables', or the sparse queues'
-    int kind = 0;   // 0 waves, 1 one source per CTA, 2 the same on a padded adjacency
+    int kind = 0;   // 0 waves, 1 one source per CTA, 2 the same on a padded adjacency, 3 all pairs
     bool operator==(const Layout& o) const {
         return n == o.n && W == o.W && blocks == o.blocks && entries == o.entries && kind == o.kind;
     }
@@ -112,7 +112,9 @@ static bcm_status region_acquire(size_t bytes, const Layout& lay, cudaStream_t s
         }
     }
     if (out->ptr) {
-        if (!(out->layout == lay)) {
+        if (lay.kind == 3) {   // all pairs: every wave writes its planes first
+            out->layout = lay;
+        } else if (!(out->layout == lay)) {
             // only the layout's own bytes must be zero; the rest is unused under it
             CU(cudaMemsetAsync(out->ptr, 0, bytes, s), "workspace clear");
             out->layout = lay;
@@ -129,7 +131,7 @@ static bcm_status region_acquire(size_t bytes, const Layout& lay, cudaStream_t s
         e = cudaMalloc(&p, bytes);
         if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");
     }
-    CU(cudaMemsetAsync(p, 0, bytes, s), "workspace clear");
+    if (lay.kind != 3) CU(cudaMemsetAsync(p, 0, bytes, s), "workspace clear");
     *out = Region{dev, p, bytes, lay};
     return BCM_OK;
 }
@@ -341,11 +343,13 @@ struct bcm_graph {
     bool preprocessed = false;
     uint32_t max_deg = 0;          // largest row length (found by preprocessing)
     uint32_t* d_lat = nullptr;     // padded adjacency of k_lattice, laid out by the first run that needs it
+    char* d_rows = nullptr;        // rows by degree descending (all pairs), laid out by the first run that needs them
     char* d_lm = nullptr;          // landmark bounds' working memory (landmark.cu)
     Aux* d_aux = nullptr;
     uint32_t* d_plain = nullptr;   // stamps [n], two vertex queues [2n]
     unsigned long long* d_far = nullptr;   // exhaustive outputs [n]
     uint32_t* d_reach = nullptr;
+    uint32_t* d_rank = nullptr;            // [n] all pairs, top-k runs: vertices that rank before
     Region slots{0, nullptr, 0, Layout{}};
     int sms = 0;
     // the run started by bcm_topk_start (or a synchronous call) until finished
@@ -397,6 +401,10 @@ struct Cfg {
     uint32_t sparse_qcap;
     int lat;                           // ... by k_lattice, rows of this many entries (0: k_sparse)
     bool walks_off;                    // an explicit hashed vertex table: sources are prefiltered at levels 0 and 1 only
+    bool all_pairs;                    // default options: farness and reach of every vertex by k_allpairs where that
+                                       // fits (ap_*, found for the run's kind: all_pairs_shape)
+    int ap_lanes;                      // its lanes (0: a choice)
+    bool ap_default;                   // no launch parameter set: a top-k run may take it
     bool landmarks;                    // ... with landmark bounds before the searches (top-k runs)
 };
 
@@ -449,6 +457,13 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
     c->sparse = !(o.flags & BCM_GRID_ONLY) &&
                 ((o.flags & BCM_SPARSE) || (!(o.flags & BCM_NO_SPARSE) && !g->directed && g->n >= 4096 &&
                                             g->max_deg <= kSparseMaxDeg));
+    // settings as the library chooses them: all pairs where that is cheap
+    c->all_pairs = !(o.flags & ~(BCM_OUT_DEVICE | BCM_NO_FOOTNOTE)) && o.shard_count <= 1 && !c->sparse &&
+                   !o.wait_limit_ns;   // (a limit of its waits is asked of the kernels that wait)
+    c->ap_lanes = (int)o.grid_lanes;
+    c->ap_default = (o.lanes == 0 || o.lanes == 64) && (o.grid_lanes == 0 || o.grid_lanes == 128) && !o.blocks &&
+                    (o.threads == 0 || o.threads == 512) && !o.heavy_words && (o.pull_div == 0 || o.pull_div == 32) &&
+                    !o.defer_words && !o.cta_table;
     // on undirected graphs whose rows fit the padded adjacency: k_lattice
     c->lat = !c->sparse || g->directed || g->n > (1u << 28) ? 0 : g->max_deg <= 4 ? 4 : g->max_deg <= 8 ? 8 : 0;
     c->landmarks = c->lat && g->n >= kLandmarkMinN &&
@@ -548,11 +563,51 @@ bcm_status ensure_aux(bcm_graph* g) {
     return BCM_OK;
 }
 
-bcm_status ensure_slots(bcm_graph* g, const Cfg& c) {
-    size_t bytes = region_bytes(g, c);
+// All pairs: slots of `clusters` clusters, then their lane words.
+struct ApShape { int W = 0, C = 0, clusters = 0; };
+constexpr size_t kApLanesBytes = 48 * sizeof(uint32_t);
+// Top-k runs take it up to this many 64-lane words gathered per level (n m /
+// 64): complete searches of a small graph from every vertex are cheaper than
+// one wave that sets a threshold and the tests behind it.  BA 2000, m = 3,
+// top-10: 0.41 ms with the seed wave, 0.14 here; BA 8000, m = 8, top-100 5.9,
+// 0.37.  With grid-wide waves (n >= 9,728) only a long list, which leaves the
+// first wave's threshold weak, pays for more (BA 16,000, m = 4: top-10 0.28 ms
+// on the grid, top-100 3.0; here 0.7).
+constexpr uint64_t kApTopkWords = 1ull << 24, kApTopkWordsMost = 1ull << 26;
+constexpr uint32_t kApLongList = 32;
+
+bool all_pairs_shape(bcm_graph* g, const Cfg& c, bool exhaustive, uint32_t k, ApShape* a) {
+    if (!c.all_pairs || g->n < 2) return false;
+    if (!exhaustive) {
+        const bool small = (uint64_t)g->n * c.grid_W < c.heavy_words;
+        const uint64_t most = small || k > kApLongList ? kApTopkWordsMost : kApTopkWords;
+        if (!c.ap_default || g->n > kAllPairsTopkN || (uint64_t)g->n * g->m / 64 > most) return false;
+    }
+    const int busy = allpairs_shape(g->n, g->sms, kAllPairsL2, exhaustive ? c.ap_lanes : 0, &a->W, &a->C, &a->clusters);
+    // a large graph whose planes leave L2 with most SMs busy stays on the grid-wide kernel
+    const uint64_t waves = ((uint64_t)g->n + 64 * a->W - 1) / (64 * a->W);
+    return busy > 0 && (busy * 4 >= g->sms * 3 || (uint64_t)a->clusters == waves);
+}
+size_t ap_bytes(bcm_graph* g, const ApShape& a) {
+    const size_t b = (size_t)a.clusters * (allpairs_slot_bytes(g->n, a.W) + kApLanesBytes);
+    const size_t sc = sorted_rows_scratch_bytes(g->n);   // before the first wave
+    return b > sc ? b : sc;
+}
+
+bcm_status ensure_slots(bcm_graph* g, const Cfg& c, const ApShape* ap = nullptr) {
+    size_t bytes = ap ? ap_bytes(g, *ap) : region_bytes(g, c);
     Layout lay = region_layout(g, c);
+    if (ap) {
+        lay = Layout{};
+        lay.n = g->n;
+        lay.W = (uint32_t)ap->W;
+        lay.blocks = (uint32_t)ap->clusters;
+        lay.kind = 3;
+    }
     if (g->slots.ptr && g->slots.bytes >= bytes) {
-        if (!(g->slots.layout == lay)) {
+        if (ap) {
+            g->slots.layout = lay;
+        } else if (!(g->slots.layout == lay)) {
             CU(cudaMemsetAsync(g->slots.ptr, 0, bytes, g->stream), "workspace clear");
             g->slots.layout = lay;
         }
@@ -924,13 +979,19 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     if (st) return st;
     if ((st = ensure_run_state(g, trace))) return st;
     const bool plain = !exhaustive && (c.flags & BCM_PLAIN);
-    if (!plain && (st = ensure_slots(g, c))) return st;
+    ApShape ap;
+    const bool pairs = !plain && all_pairs_shape(g, c, exhaustive, k, &ap);
+    if (!plain && (st = ensure_slots(g, c, pairs ? &ap : nullptr))) return st;
     if (!plain && c.lat && !g->d_lat) {
         CU(buf_get_t(&g->d_lat, (size_t)g->n * c.lat * sizeof(uint32_t)), "padded adjacency allocation");
         if (launch_lattice_rows(g->d_rp, g->d_col, g->n, c.lat, g->d_lat, s))
             return fail(BCM_ERR_CUDA, "padded adjacency kernel: %s", cudaGetErrorString(cudaGetLastError()));
     }
-    if (exhaustive && !g->d_far) {
+    const bool lay_rows = pairs && !g->d_rows;
+    if (lay_rows) CU(buf_get_t(&g->d_rows, sorted_rows_bytes(g->n, g->m)), "row allocation");
+    if (pairs && !exhaustive && !g->d_rank)
+        CU(buf_get_t(&g->d_rank, (size_t)g->n * sizeof(uint32_t)), "rank allocation");
+    if ((exhaustive || pairs) && !g->d_far) {
         CU(buf_get_t(&g->d_far, (size_t)g->n * sizeof(uint64_t) + 256), "output allocation");
         CU(buf_get_t(&g->d_reach, (size_t)g->n * sizeof(uint32_t) + 256), "output allocation");
     }
@@ -984,6 +1045,30 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         for (uint32_t it = 0; it < g->n && rc == 0; ++it)
             rc = launch_plain_source(p, it, g->d_plain, g->d_plain + g->n, blocks, 256, s);
         cudaEventRecord(g->ev[1], s);
+    } else if (pairs) {
+        AllPairs a;
+        a.n = g->n;
+        if (lay_rows)   // the planes' memory serves as scratch
+            rc = launch_sorted_rows(g->d_rp, g->d_col, g->d_order, g->n, g->m, g->d_rows, g->slots.ptr, s);
+        sorted_rows_use(&a, g->d_rows, g->m, g->d_order);
+        a.grp = g->d_rp;
+        a.rrp = p.g.rrp;
+        a.rcol = p.g.rcol;
+        a.slots = (char*)g->slots.ptr;
+        a.slot_stride = allpairs_slot_bytes(g->n, ap.W);
+        a.lanes = (uint32_t*)(a.slots + (size_t)ap.clusters * a.slot_stride);
+        a.far = g->d_far;
+        a.reach = g->d_reach;
+        a.stats = p.stats;
+        CU(cudaMemsetAsync(g->d_far, 0, (size_t)g->n * sizeof(uint64_t), s), "output clear");
+        CU(cudaMemsetAsync(g->d_reach, 0, (size_t)g->n * sizeof(uint32_t), s), "output clear");
+        if (rc == 0) rc = launch_allpairs(a, ap.W, ap.C, ap.clusters, s);
+        if (!exhaustive && rc == 0) {
+            CU(cudaMemsetAsync(g->d_rank, 0, (size_t)g->n * sizeof(uint32_t), s), "rank clear");
+            rc = launch_rank_topk(g->d_far, g->d_reach, g->n, g->d_rank, p.topk, s);
+        }
+        cudaEventRecord(g->ev[1], s);
+        cudaEventRecord(g->ev[2], s);
     } else {
         // grid-wide waves while they are heavy (every wave for exhaustive
         // runs), then per-CTA waves from wherever the grid kernel left head.
@@ -1142,7 +1227,7 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     g->pend.active = true;
     g->pend.exhaustive = exhaustive;
     g->pend.plain = plain;
-    g->pend.sparse = !plain && c.sparse;
+    g->pend.sparse = !plain && !pairs && c.sparse;
     g->pend.lat = plain ? 0 : c.lat;
     g->pend.kk = k < n_src ? k : n_src;
     g->pend.flags = c.flags;
@@ -1347,7 +1432,8 @@ bcm_status bcm_graph_destroy(bcm_graph_t g) {
     else cudaDeviceSynchronize();
     for (void* b : {(void*)g->d_rp, (void*)g->d_col, (void*)g->d_order, (void*)g->d_aux, (void*)g->d_plain,
                     (void*)g->d_far, (void*)g->d_reach, (void*)g->d_rrp, (void*)g->d_rcol, (void*)g->d_trace,
-                    (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lat, (void*)g->d_lm})
+                    (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lat, (void*)g->d_lm, (void*)g->d_rank,
+                    (void*)g->d_rows})
         buf_put(b);
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -1572,8 +1658,9 @@ bcm_status bcm_graph_trim(bcm_graph_t g) {
     CU(g->stream ? cudaStreamSynchronize(g->stream) : cudaDeviceSynchronize(), "synchronize");
     region_release(g->slots, true);
     for (void* b : {(void*)g->d_plain, (void*)g->d_far, (void*)g->d_reach, (void*)g->d_trace, (void*)g->d_defer,
-                    (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lm})
+                    (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lm, (void*)g->d_rank})
         buf_put(b);
+    g->d_rank = nullptr;
     g->d_lm = nullptr;
     g->d_surv = nullptr;
     g->d_defer = nullptr;
@@ -1786,7 +1873,14 @@ uint64_t bcm_workspace_bytes(bcm_graph_t g, const bcm_options* opt) {
     if (!g->preprocessed && preprocess(g, nullptr) != BCM_OK) return 0;   // the default kernels depend on it
     Cfg c;
     if (resolve(g, opt, &c)) return 0;
-    return (uint64_t)region_bytes(g, c) + sizeof(Aux) + (uint64_t)g->n * (8 + 4 * c.lat) + walks_bytes(g->n) +
+    size_t region = region_bytes(g, c);
+    for (bool all : {false, true}) {
+        ApShape ap;
+        if (!all_pairs_shape(g, c, all, 1024, &ap)) continue;
+        const size_t b = ap_bytes(g, ap) + (size_t)g->n * 16 + sorted_rows_bytes(g->n, g->m);
+        region = b > region ? b : region;
+    }
+    return (uint64_t)region + sizeof(Aux) + (uint64_t)g->n * (8 + 4 * c.lat) + walks_bytes(g->n) +
            (c.landmarks ? landmark_bytes(g->n) : 0);
 }
 

@@ -258,6 +258,35 @@ int launch_landmarks(const WaveParams& p, const Landmarks& L, int rw, uint32_t n
 int launch_landmark_filter(const WaveParams& p, const Landmarks& L, const uint32_t* order, uint32_t first,
                            uint32_t n_src, cudaStream_t s);
 
+// ---- allpairs.cu: farness and reach of every vertex, the lanes of a wave being targets
+struct AllPairs {
+    uint32_t n;
+    const uint32_t *rp, *col;      // out-arcs, rows by degree descending (launch_sorted_rows) ...
+    const uint32_t* vertex;        // ... row i that of vertex[i]; NULL: row i is vertex i, in any order
+    const uint32_t* pos;           // the row of each vertex
+    const uint32_t* grp;           // the graph's own offsets
+    const uint32_t *rrp, *rcol;    // its in-arcs (NULL: not there)
+    char* slots;                   // one per cluster, allpairs_slot_bytes apart
+    size_t slot_stride;
+    uint32_t* lanes;               // [clusters][48]
+    unsigned long long* far;       // [n] zeroed
+    uint32_t* reach;               // [n] zeroed
+    unsigned long long* stats;     // [ST_COUNT]
+};
+constexpr size_t kAllPairsL2 = 130ull << 20;   // (R-MAT 2^16: 129 MB at 256 lanes 12.2 ms, 70 MB at 128 13.9)
+constexpr uint32_t kAllPairsTopkN = 16384;
+size_t allpairs_slot_bytes(uint32_t n, int W);
+int allpairs_shape(uint32_t n, int sms, size_t budget, int lanes, int* W, int* C, int* clusters);
+size_t sorted_rows_bytes(uint32_t n, uint64_t m);
+size_t sorted_rows_scratch_bytes(uint32_t n);
+int launch_sorted_rows(const uint32_t* grp, const uint32_t* gcol, const uint32_t* order, uint32_t n, uint64_t m,
+                       void* rows, void* scratch, cudaStream_t s);
+void sorted_rows_use(AllPairs* a, const void* rows, uint64_t m, const uint32_t* order);
+int launch_allpairs(const AllPairs& p, int W, int C, int clusters, cudaStream_t s);
+// the top-k from every vertex's farness and reach (rank: [n] zeroed)
+int launch_rank_topk(const unsigned long long* far, const uint32_t* reach, uint32_t n, uint32_t* rank, const TopK& T,
+                     cudaStream_t s);
+
 // launch bookkeeping (api.cu)
 void note_launch(int count = 1);
 // sets the calling thread's bcm_last_error() message (api.cu)

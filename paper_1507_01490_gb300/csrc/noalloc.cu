@@ -26,7 +26,9 @@
 
 namespace bcm {
 
-// 64 MiB: the CSR offsets narrowed to 32 bits, a source order, and the
+// 64 MiB: the CSR offsets narrowed to 32 bits, then either the planes of as
+// many waves of k_allpairs as fit (and, where there is room, its sorted rows),
+// or, on graphs too large for most SMs to have one, a source order and the
 // per-CTA wave slots (44 bytes per vertex each) for as many CTAs as fit.
 constexpr size_t kNoAllocBytes = 64ull << 20;
 constexpr uint32_t kNoAllocMaxN = 1250000;   // at least one CTA slot (44 bytes per vertex) fits
@@ -117,6 +119,67 @@ extern "C" bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uin
     uint32_t* rp32 = (uint32_t*)(p + kHeaderBytes);
     uint32_t* order = (uint32_t*)((char*)rp32 + al256(((size_t)n + 1) * 4));
     char* slots = (char*)order + al256((size_t)n * 4);
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess || sms <= 0) {
+        char buf[256];
+        snprintf(buf, sizeof(buf), "bcm_farness_all_noalloc: reading the SM count failed: %s", cudaGetErrorString(e));
+        return noalloc_fail(BCM_ERR_CUDA, buf);
+    }
+    {
+        // all pairs: header | offsets | [order | sorted rows] | lane words | slots
+        const size_t lane_bytes = al256((size_t)sms * 48 * sizeof(uint32_t));
+        const size_t off = kHeaderBytes + al256(((size_t)n + 1) * 4);
+        const size_t rows = al256((size_t)n * 4) + sorted_rows_bytes(n, m);
+        // (laying the rows out takes ten launches: 0.1 ms, as much as all of n = 1000)
+        const bool sorted = n >= 8192 && off + rows + lane_bytes + al256(degree_order_scratch_bytes(n)) <= kNoAllocBytes / 2;
+        const size_t used = off + lane_bytes + (sorted ? rows : 0);
+        int W = 0, C = 0, clusters = 0;
+        const int busy = used < kNoAllocBytes ? allpairs_shape(n, sms, kNoAllocBytes - used, 0, &W, &C, &clusters) : 0;
+        const uint64_t waves = W ? ((uint64_t)n + 64 * W - 1) / (64 * W) : 0;
+        if (busy > 0 && (busy * 4 >= sms * 3 || (uint64_t)clusters == waves)) {
+            if (cudaMemsetAsync(hdr, 0, sizeof(NoAllocHeader), s) != cudaSuccess)
+                return noalloc_fail(BCM_ERR_CUDA, "clearing the working array failed");
+            if (launch_validate(row_ptr, col, n, m, &hdr->csr_err, s) || launch_narrow_offsets(row_ptr, rp32, n, s))
+                return noalloc_fail(BCM_ERR_CUDA, "CSR check kernels failed to launch");
+            int cerr = 0;
+            // a malformed CSR must not reach the other kernels
+            if (cudaMemcpyAsync(&cerr, &hdr->csr_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess)
+                return noalloc_fail(BCM_ERR_CUDA, "CSR check failed");
+            if (cerr)
+                return noalloc_fail(BCM_ERR_INVALID, "malformed CSR: row_ptr must rise from 0 to m and every col < n");
+            char* lay = (char*)base + off + (sorted ? rows : 0);
+            AllPairs a;
+            a.n = n;
+            a.rp = rp32;
+            a.col = col;
+            a.vertex = nullptr;
+            a.pos = nullptr;
+            a.grp = rp32;
+            a.rrp = nullptr;    // the graph may be directed, and its in-arcs are not given
+            a.rcol = nullptr;
+            a.lanes = (uint32_t*)lay;
+            a.slots = lay + lane_bytes;
+            a.slot_stride = allpairs_slot_bytes(n, W);
+            a.far = (unsigned long long*)farness;
+            a.reach = reach;
+            a.stats = hdr->stats;
+            if (sorted) {
+                char* rbuf = (char*)order + al256((size_t)n * 4);
+                if (launch_degree_order(rp32, n, order, a.slots, degree_order_scratch_bytes(n), s) ||
+                    launch_sorted_rows(rp32, col, order, n, m, rbuf, a.slots, s))
+                    return noalloc_fail(BCM_ERR_CUDA, "laying out the rows failed");
+                sorted_rows_use(&a, rbuf, m, order);
+            }
+            if (cudaMemsetAsync(farness, 0, (size_t)n * sizeof(uint64_t), s) != cudaSuccess ||
+                cudaMemsetAsync(reach, 0, (size_t)n * sizeof(uint32_t), s) != cudaSuccess)
+                return noalloc_fail(BCM_ERR_CUDA, "clearing the outputs failed");
+            if (launch_allpairs(a, W, C, clusters, s)) return noalloc_fail(BCM_ERR_CUDA, "wave kernel launch failed");
+            if (cudaStreamSynchronize(s) != cudaSuccess) return noalloc_fail(BCM_ERR_CUDA, "wave kernel failed");
+            return BCM_OK;
+        }
+    }
     const size_t fixed = noalloc_fixed_bytes(n);
     const size_t sb = slot_bytes(n, 1);
     const int per = cta_blocks_per_sm(1, 512);
@@ -125,13 +188,6 @@ extern "C" bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uin
         char buf[256];
         snprintf(buf, sizeof(buf), "bcm_farness_all_noalloc: the occupancy query of the wave kernel failed: %s",
                  cudaGetErrorString(oe));
-        return noalloc_fail(BCM_ERR_CUDA, buf);
-    }
-    int sms = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess || sms <= 0) {
-        char buf[256];
-        snprintf(buf, sizeof(buf), "bcm_farness_all_noalloc: reading the SM count failed: %s", cudaGetErrorString(e));
         return noalloc_fail(BCM_ERR_CUDA, buf);
     }
     size_t fit = (kNoAllocBytes - fixed) / sb;
