@@ -343,6 +343,7 @@ struct bcm_graph {
     bool preprocessed = false;
     uint32_t max_deg = 0;          // largest row length (found by preprocessing)
     uint32_t* d_lat = nullptr;     // padded adjacency of k_lattice, laid out by the first run that needs it
+    bool walks_base = false;       // d_walk is filled
     char* d_rows = nullptr;        // rows by degree descending (all pairs), laid out by the first run that needs them
     char* d_lm = nullptr;          // landmark bounds' working memory (landmark.cu)
     Aux* d_aux = nullptr;
@@ -635,7 +636,8 @@ double ms_since(std::chrono::steady_clock::time_point t0) {
 // ------------------------------------------------------ preprocessing
 bcm_status ensure_run_state(bcm_graph* g, bool trace);
 
-bcm_status preprocess(bcm_graph* g, double* ms) {
+// topk: called by a top-k run, which may want the prefilter's counts.
+bcm_status preprocess(bcm_graph* g, double* ms, bool topk = false) {
     if (g->preprocessed) return BCM_OK;
     cudaStream_t s = g->stream;
     const uint32_t n = g->n;
@@ -696,19 +698,23 @@ bcm_status preprocess(bcm_graph* g, double* ms) {
         K.c[2] = (uint32_t*)((char*)g->d_walk + nb);
         K.heavy_n = (uint32_t*)(d_simple + 16);
         K.heavy = (uint32_t*)(d_scr2 + dos + scs + 256);
+        // (a run that finds them missing makes them; lattices and the smallest
+        // graphs hardly ever want them)
+        const bool walks = topk && n >= 9728 && (g->directed || g->max_deg > kSparseMaxDeg);
         const bool walks_after = !g->directed && n <= 65536;
-        if (!walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, !g->directed, g->aux)) {
+        g->walks_base = walks;
+        if (walks && !walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, !g->directed, g->aux)) {
             st = fail(BCM_ERR_CUDA, "walk counts: %s", cudaGetErrorString(cudaGetLastError()));
             break;
         }
         if (!g->directed) {
             uint32_t* parent = g->d_comp;
             uint32_t* size = (uint32_t*)d_scr;
-            if (launch_cc_reach(g->d_rp, g->d_col, n, parent, size, g->d_xlo, g->d_xhi, d_err, s)) {
+            if (launch_cc_reach(g->d_rp, g->d_col, n, g->max_deg, parent, size, g->d_xlo, g->d_xhi, d_err, s)) {
                 st = fail(BCM_ERR_CUDA, "component kernels: %s", cudaGetErrorString(cudaGetLastError()));
                 break;
             }
-            if (walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, true, s)) {
+            if (walks && walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, true, s)) {
                 st = fail(BCM_ERR_CUDA, "walk counts: %s", cudaGetErrorString(cudaGetLastError()));
                 break;
             }
@@ -1133,7 +1139,9 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
             uint32_t* const left_n = g->d_aux->walk_left;
             WaveParams pf = p;
             pf.stats = g->d_aux->stats;
-            rc = launch_prefilter(pf, K, !g->directed, K.list[0], left_n, s);
+            if (!g->walks_base && launch_walk_base(g->d_rp, g->d_col, g->n, K, !g->directed, s)) rc = -1;
+            g->walks_base = rc == 0;
+            if (rc == 0) rc = launch_prefilter(pf, K, !g->directed, K.list[0], left_n, s);
             pc.sources = K.list[0];
             pc.head = &g->d_aux->head3;
             pc.n_end = 0;
@@ -1499,7 +1507,7 @@ bcm_status bcm_topk_start(bcm_graph_t g, uint32_t k, const bcm_options* opt, uin
     if (k < 1 || k > 1024) return fail(BCM_ERR_INVALID, "k = %u: must be in 1..1024", k);
     if (!ids || !farness || !reach) return fail(BCM_ERR_INVALID, "output pointer is NULL");
     double pms = 0;
-    bcm_status st = preprocess(g, &pms);
+    bcm_status st = preprocess(g, &pms, true);
     if (st) return st;
     Cfg c;
     if ((st = resolve(g, opt, &c))) return st;
