@@ -115,7 +115,8 @@ typedef enum {
  * atomics). */
 typedef struct {
     uint32_t lanes;           /* sources per per-CTA wave: 64, 128 or 256; 0 = 64 */
-    uint32_t grid_lanes;      /* sources per grid-wide wave: 64, 128 or 256; 0 = 128 */
+    uint32_t grid_lanes;      /* sources per grid-wide wave: 64, 128 or 256; 0 = 128, and 256 while more
+                                 than 512 are queued behind the prefilter or from the start if k > 32 */
     uint32_t flags;           /* BCM_* flags above */
     uint32_t blocks;          /* CTAs of the per-CTA kernel; 0 = all that fit on the GPU, at most
                                  one per wave of sources (ceil(n / lanes)).  Each holds a slot of

@@ -391,6 +391,7 @@ constexpr uint64_t kDefaultLimitNs = 20ull * 1000 * 1000 * 1000;
 
 struct Cfg {
     int W, threads, blocks, grid_W, grid_blocks;
+    int wide_blocks;                   // grid CTAs at 256 lanes, where the library chooses the lanes (0: the caller did)
     uint32_t pull_div;
     uint64_t heavy_words;
     uint64_t defer_words;
@@ -499,6 +500,7 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
     int gb = max_coop_blocks(0, c->grid_W, 512);
     if (gb < 1) return fail(BCM_ERR_CUDA, "grid wave kernel does not fit on an SM");
     c->grid_blocks = gb;
+    c->wide_blocks = o.grid_lanes ? 0 : max_coop_blocks(0, 4, 512);
     c->heavy_words = o.heavy_words ? o.heavy_words : (uint64_t)gb * 16 * 4;   // 4 words per warp and level
     c->pull_div = (c->flags & BCM_NO_PULL) ? 0u : o.pull_div;   // 0: per-mode default below
     c->defer_words = (c->flags & BCM_NO_DEFER) ? 0 : (o.defer_words ? o.defer_words : c->heavy_words);
@@ -576,6 +578,13 @@ constexpr size_t kApLanesBytes = 48 * sizeof(uint32_t);
 // on the grid, top-100 3.0; here 0.7).
 constexpr uint64_t kApTopkWords = 1ull << 24, kApTopkWordsMost = 1ull << 26;
 constexpr uint32_t kApLongList = 32;
+// Grid-wide waves take 256 lanes while this many sources are queued, 128 after
+// (and in the first wave of a short list): a wave of 256 costs 1.7 times one
+// of 128, so it pays once a third one would follow.  128 lanes -> this: R-MAT
+// 2^20 top-10 15.1 -> 13.1 ms, BA 150,000 m = 3 top-100 13.4 -> 7.4, Chung-Lu
+// 200,003 top-100 0.72 -> 0.63; Chung-Lu 2^20 top-10 stays at 1.2 (256 lanes
+// throughout: 1.38).
+constexpr uint32_t kWideLeft = 512;
 
 bool all_pairs_shape(bcm_graph* g, const Cfg& c, bool exhaustive, uint32_t k, ApShape* a) {
     if (!c.all_pairs || g->n < 2) return false;
@@ -1105,7 +1114,10 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
                             !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY));
         if (grid) {
             // as many waves as give k entries come before the prefilter
-            const uint32_t lanes = 64u * (uint32_t)c.grid_W;
+            // (a long list: 256 lanes, so that the first wave already holds
+            // more than k sources)
+            const bool wide = filter && c.wide_blocks && k > kApLongList;
+            const uint32_t lanes = wide ? 256u : 64u * (uint32_t)c.grid_W;
             p.max_grid_waves = filter ? (k + lanes - 1) / lanes : 0xffffffffu;
             p.light = filter ? &g->d_aux->light : nullptr;
             p.walk_want = filter ? &g->d_aux->walk_want : nullptr;
@@ -1114,7 +1126,8 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
             // default measured per level on the Chung-Lu and R-MAT workloads:
             // pull wins once the frontier's out-arcs reach about n*W/32
             p.pull_div = (c.flags & BCM_NO_PULL) ? 0u : (c.pull_div ? c.pull_div : 32u);
-            rc = launch_grid_waves(p, c.grid_W, c.grid_blocks, 512, s);
+            rc = wide ? launch_grid_waves(p, 4, c.wide_blocks, 512, s)
+                      : launch_grid_waves(p, c.grid_W, c.grid_blocks, 512, s);
         }
         // a graph too small for grid-wide waves: one CTA first runs the
         // first wave alone (the highest-degree sources), so the threshold
@@ -1153,7 +1166,12 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
                 pc.pick = c.flags & BCM_TRACE_LANES ? 0u : 1u;
                 pc.walks = K;
                 pc.walk_want = nullptr;
-                rc = launch_grid_waves(pc, c.grid_W, c.grid_blocks, 512, s);
+                if (c.wide_blocks) {
+                    WaveParams pw = pc;
+                    pw.min_left = kWideLeft;
+                    rc = launch_grid_waves(pw, 4, c.wide_blocks, 512, s);
+                }
+                if (rc == 0) rc = launch_grid_waves(pc, c.grid_W, c.grid_blocks, 512, s);
                 pf = pc;
                 pf.stats = g->d_aux->stats;
                 if (rc == 0) rc = launch_refilter(pf, K, !g->directed, K.list[1], left_n + 1, s);

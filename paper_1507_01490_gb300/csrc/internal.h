@@ -151,6 +151,7 @@ struct WaveParams {
     uint32_t* wave_src;      // [256]
     uint32_t* wave_n;
     uint32_t pick, undirected;
+    uint32_t min_left;       // the launch ends once fewer sources than this are queued (0: never)
     uint32_t* walk_want;     // receives, when the launch ends, how many walk counts the prefilter wants
     Walks walks;
     uint32_t* light;         // grid-wide kernel: set when a narrow wave ended it; set on entry: nothing to do

@@ -1976,6 +1976,10 @@ __device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, co
     const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
     __syncthreads();
     u32 base = vload(p.head), cnt = 0;
+    if (p.min_left && (base >= n_end || n_end - base < p.min_left)) {   // left to a narrower launch
+        if (tid == 0) vstore(p.wave_n, 0u);
+        return;
+    }
     const int use = p.pick ? (int)__ldcg(p.walks.want) : 0;
     while (cnt < L && base < n_end) {
         const u32 pos = base + tid;
