@@ -740,13 +740,14 @@ def main():
     h2d = int(g.row_ptr.nbytes + g.col.nbytes)
     d2h = int(kk * (4 + 8 + 4))
 
-    # roofline of the dominant kernel: the grid-wide or the per-CTA wave kernel,
-    # whichever took longer (one launch each per step)
+    # roofline of the dominant phase: the grid-wide waves (with the prefilter
+    # between them) or the per-CTA / one-source kernel, whichever took longer
     peak, peak_kind = load_peaks()
     if st["seed_ms"] >= st["wave_ms"]:
         kname, kms, kbytes = "k_wave_grid", st["seed_ms"], st["grid_bytes"]
     else:
-        kname, kms, kbytes = ("k_sparse" if st["sparse"] else "k_wave_cta"), st["wave_ms"], st["wave_bytes"]
+        one_source = "k_lattice" if not g.directed and int(g.degrees().max()) <= 8 else "k_sparse"
+        kname, kms, kbytes = (one_source if st["sparse"] else "k_wave_cta"), st["wave_ms"], st["wave_bytes"]
     achieved = kbytes / (kms / 1e3) / 1e9 if kms > 0 else None
     src_hash = kernel_source_hash()
     traffic = profile_traffic(kname, src_hash, args.workload)
@@ -821,7 +822,7 @@ def main():
         "config": {"workload": "%s: %s" % (args.workload, WORKLOADS[args.workload]), "n": g.n, "m_arcs": g.m,
                    "k": k, "lanes": par["lanes"] or 64, "grid_lanes": par["grid_lanes"] or 128,
                    "pull_div": par["pull_div"] or 32, "threads": par["threads"] or (256 if st["sparse"] else 512),
-                   "per_cta_kernel": "k_sparse (one source per CTA)" if st["sparse"] else "k_wave_cta (bit lanes)",
+                   "per_cta_kernel": "one source per CTA" if st["sparse"] else "k_wave_cta (bit lanes)",
                    "launch_parameters": ("autotuned for this graph (%.2f s, outside the timed region)" % tuning_s)
                    if tuned else "library defaults" if not (args.lanes or args.threads or args.grid_lanes)
                    else "command line",

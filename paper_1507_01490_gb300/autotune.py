@@ -6,7 +6,8 @@ trial); only the time does.  So each graph gets the setting that ran
 fastest on it:
 
   lanes        sources per per-CTA wave (64, 128, 256)
-  grid_lanes   sources per grid-wide wave (64, 128, 256)
+  grid_lanes   sources per grid-wide wave (64, 128, 256; 0: the library's choice,
+               128 or 256 by what is queued)
   pull_div     the push/pull switch: a grid level is pulled once its
                frontier's out-arcs reach n*W/pull_div
   threads      the per-CTA kernel's block shape (256, 512, 1024 threads)
@@ -33,12 +34,12 @@ import numpy as np
 from . import bcm
 
 SPACE = {
-    "grid_lanes": (128, 64, 256),
+    "grid_lanes": (0, 128, 64, 256),
     "pull_div": (32, 8, 16, 64, 128),
     "lanes": (64, 128, 256),
     "threads": (512, 256, 1024),
 }
-DEFAULTS = {"grid_lanes": 128, "pull_div": 32, "lanes": 64, "threads": 512}
+DEFAULTS = {"grid_lanes": 0, "pull_div": 32, "lanes": 64, "threads": 512}
 PER_CTA = {"auto": 0, "bitlanes": bcm.BCM_NO_SPARSE, "sparse": bcm.BCM_SPARSE}
 KERNEL_MAX_DEG = 64   # graphs with a larger degree keep the library's choice
 KERNEL_TRIAL_MS = 200.0   # ... and so do graphs whose default run takes longer

@@ -344,6 +344,8 @@ struct bcm_graph {
     uint32_t max_deg = 0;          // largest row length (found by preprocessing)
     uint32_t* d_lat = nullptr;     // padded adjacency of k_lattice, laid out by the first run that needs it
     bool walks_base = false;       // d_walk is filled
+    bool rows_ready = false;       // d_rows is laid out
+    bool lat_ready = false;        // d_lat is
     char* d_rows = nullptr;        // rows by degree descending (all pairs), laid out by the first run that needs them
     char* d_lm = nullptr;          // landmark bounds' working memory (landmark.cu)
     Aux* d_aux = nullptr;
@@ -578,6 +580,7 @@ constexpr size_t kApLanesBytes = 48 * sizeof(uint32_t);
 // on the grid, top-100 3.0; here 0.7).
 constexpr uint64_t kApTopkWords = 1ull << 24, kApTopkWordsMost = 1ull << 26;
 constexpr uint32_t kApLongList = 32;
+constexpr uint64_t kApMostArcs = 1ull << 28;   // its copy of the rows: 1 GB
 // Grid-wide waves take 256 lanes while this many sources are queued, 128 after
 // (and in the first wave of a short list): a wave of 256 costs 1.7 times one
 // of 128, so it pays once a third one would follow.  128 lanes -> this: R-MAT
@@ -587,7 +590,7 @@ constexpr uint32_t kApLongList = 32;
 constexpr uint32_t kWideLeft = 512;
 
 bool all_pairs_shape(bcm_graph* g, const Cfg& c, bool exhaustive, uint32_t k, ApShape* a) {
-    if (!c.all_pairs || g->n < 2) return false;
+    if (!c.all_pairs || g->n < 2 || g->m > kApMostArcs) return false;
     if (!exhaustive) {
         const bool small = (uint64_t)g->n * c.grid_W < c.heavy_words;
         const uint64_t most = small || k > kApLongList ? kApTopkWordsMost : kApTopkWords;
@@ -995,15 +998,20 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     if ((st = ensure_run_state(g, trace))) return st;
     const bool plain = !exhaustive && (c.flags & BCM_PLAIN);
     ApShape ap;
-    const bool pairs = !plain && all_pairs_shape(g, c, exhaustive, k, &ap);
+    bool pairs = !plain && all_pairs_shape(g, c, exhaustive, k, &ap);
+    if (pairs && !g->d_rows && buf_get_t(&g->d_rows, sorted_rows_bytes(g->n, g->m)) != cudaSuccess) {
+        cudaGetLastError();   // no room for its rows: the wave kernels need none
+        g->d_rows = nullptr;
+        pairs = false;
+    }
     if (!plain && (st = ensure_slots(g, c, pairs ? &ap : nullptr))) return st;
-    if (!plain && c.lat && !g->d_lat) {
-        CU(buf_get_t(&g->d_lat, (size_t)g->n * c.lat * sizeof(uint32_t)), "padded adjacency allocation");
+    if (!plain && c.lat && !g->lat_ready) {
+        if (!g->d_lat)
+            CU(buf_get_t(&g->d_lat, (size_t)g->n * c.lat * sizeof(uint32_t)), "padded adjacency allocation");
         if (launch_lattice_rows(g->d_rp, g->d_col, g->n, c.lat, g->d_lat, s))
             return fail(BCM_ERR_CUDA, "padded adjacency kernel: %s", cudaGetErrorString(cudaGetLastError()));
+        g->lat_ready = true;
     }
-    const bool lay_rows = pairs && !g->d_rows;
-    if (lay_rows) CU(buf_get_t(&g->d_rows, sorted_rows_bytes(g->n, g->m)), "row allocation");
     if (pairs && !exhaustive && !g->d_rank)
         CU(buf_get_t(&g->d_rank, (size_t)g->n * sizeof(uint32_t)), "rank allocation");
     if ((exhaustive || pairs) && !g->d_far) {
@@ -1063,8 +1071,9 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     } else if (pairs) {
         AllPairs a;
         a.n = g->n;
-        if (lay_rows)   // the planes' memory serves as scratch
+        if (!g->rows_ready)   // the planes' memory serves as scratch
             rc = launch_sorted_rows(g->d_rp, g->d_col, g->d_order, g->n, g->m, g->d_rows, g->slots.ptr, s);
+        g->rows_ready = rc == 0;
         sorted_rows_use(&a, g->d_rows, g->m, g->d_order);
         a.grp = g->d_rp;
         a.rrp = p.g.rrp;
@@ -1110,8 +1119,13 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         // on a simple graph, sources are tested at levels 0 to 2 from counts of
         // walks alone as soon as a threshold exists -- after the first grid
         // waves, or the seed wave -- and only the others are searched
-        const bool filter = g->simple && !exhaustive && !c.sparse &&
-                            !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY));
+        bool filter = g->simple && !exhaustive && !c.sparse &&
+                      !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY));
+        if (filter && !g->d_surv && buf_get_t(&g->d_surv, walks_bytes(g->n)) != cudaSuccess) {
+            cudaGetLastError();   // no room: the waves do without
+            g->d_surv = nullptr;
+            filter = false;
+        }
         if (grid) {
             // as many waves as give k entries come before the prefilter
             // (a long list: 256 lanes, so that the first wave already holds
@@ -1143,10 +1157,6 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         }
         WaveParams pc = p;
         if (filter && (grid || seed) && rc == 0) {
-            if (!g->d_surv) {
-                cudaError_t e = buf_get_t(&g->d_surv, walks_bytes(g->n));
-                if (e != cudaSuccess) { cudaStreamSynchronize(s); return cuda_fail(e, "prefilter allocation"); }
-            }
             Walks K = carve_walks(g);
             K.off = c.walks_off ? 1u : 0u;
             uint32_t* const left_n = g->d_aux->walk_left;
@@ -1182,13 +1192,15 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         }
         pc.stats = g->d_aux->stats;
         cudaEventRecord(g->ev[1], s);
-        if (rc == 0 && c.landmarks && !exhaustive) {
+        bool landmarks = c.landmarks && !exhaustive;
+        if (landmarks && !g->d_lm && buf_get_t(&g->d_lm, landmark_bytes(g->n)) != cudaSuccess) {
+            cudaGetLastError();   // no room: the searches do without
+            g->d_lm = nullptr;
+            landmarks = false;
+        }
+        if (rc == 0 && landmarks) {
             // sources by landmark bound; the most central ones first, which
             // sets the threshold; the others if no bound stops them
-            if (!g->d_lm) {
-                cudaError_t e = buf_get_t(&g->d_lm, landmark_bytes(g->n));
-                if (e != cudaSuccess) { cudaStreamSynchronize(s); return cuda_fail(e, "landmark allocation"); }
-            }
             const Landmarks L = landmark_carve(g->d_lm, g->n);
             uint32_t* order = nullptr;
             rc = launch_landmarks(pc, L, c.lat, n_src, &order, s);
