@@ -84,8 +84,8 @@ __device__ __noinline__ long long cut_limit(const ThrCache& t, u32 x, u32 v) {
     return lim > (unsigned __int128)never ? never : (long long)lim;
 }
 
-// A completed source of a top-k run: into the shared top-k if it ranks
-// before the threshold.  While another CTA holds the lock the threshold is
+// A completed source of a top-k run: into the shared top-k unless the
+// threshold ranks before it.  While another CTA holds the lock the threshold is
 // read again: it only rises, and most waiters then have nothing to insert
 // (before a threshold exists, thousands of sources complete together).
 __device__ __noinline__ void lattice_complete(const WaveParams& p, ThrCache& t, u32 v, u64 f, u32 r) {
@@ -94,7 +94,7 @@ __device__ __noinline__ void lattice_complete(const WaveParams& p, ThrCache& t, 
     const u64 t0 = global_ns();
     u32 ns = 32;
     for (;;) {
-        if (t.valid && !ranks_before(N, F, v, t.N, t.F, t.id)) return;
+        if (t.valid && ranks_before(t.N, t.F, t.id, N, F, v)) return;   // (equal: an offered key that is its own)
         if (atomicCAS(p.topk.lock, 0u, 1u) == 0u) break;
         if (global_ns() - t0 > p.lock_limit_ns) { atomicOr(p.err, DEV_ERR_LOCK_TIMEOUT); return; }
         __nanosleep(ns);

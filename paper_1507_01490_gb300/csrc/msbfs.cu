@@ -906,7 +906,7 @@ __device__ inline void pull_clear(const u32* list, u32 cnt, u64* Fcur, u32 gtid,
 }
 
 // Completed lanes: exhaustive runs write (f, r) by vertex id; top-k runs
-// merge the ones that beat the cached k-th key into the shared top-k, under
+// merge the ones that the cached k-th key does not rank before into the shared top-k, under
 // the lock, with the whole block: the held entries (best first) are copied
 // to shared memory, the new ones ranked among themselves, every entry's
 // final place found by binary search in the other list, and the first k
@@ -930,7 +930,8 @@ __device__ __noinline__ void flush_completions(const WaveParams& p, const u32* c
         for (u32 i = 0; i < nc && !any; ++i) {
             u64 N, F;
             score_key(cf[i], cr[i], N, F);
-            any = ranks_before(N, F, cid[i], thr.N, thr.F, thr.id);
+            // (equal: the offered key is this source's own, and the run holds it only if merged)
+            any = !ranks_before(thr.N, thr.F, thr.id, N, F, cid[i]);
         }
         *s_go = any && lock_acquire(T.lock, p.lock_limit_ns, p.err);
     }
@@ -1220,8 +1221,8 @@ __device__ __forceinline__ void filter_sources(const WaveParams& p, const Walks&
             if (p.trace_lanes) lane_level(p, v, 0, 0, 1, deg);
             if (deg == 0) {
                 // R(v) = {v}: complete with key (0, 1); it only goes on (to be
-                // merged by a wave) if it ranks before the k-th
-                if (!ranks_before(0, 1, v, thr.N, thr.F, thr.id)) {
+                // merged by a wave) if the k-th does not rank before it
+                if (ranks_before(thr.N, thr.F, thr.id, 0, 1, v)) {
                     stays = false;
                     ++ndone;
                     if (p.trace_lanes) lane_end(p, v, 0, 0, 1, false);
@@ -1992,7 +1993,7 @@ __device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, co
                 deg = p.walks.c[1][v];
                 const u32 c2 = p.walks.c[2][v], xlo = __ldg(&p.g.xlo[v]), xhi = __ldg(&p.g.xhi[v]);
                 if (deg == 0) {
-                    keep = ranks_before(0, 1, v, thr.N, thr.F, thr.id);
+                    keep = !ranks_before(thr.N, thr.F, thr.id, 0, 1, v);
                     done = !keep;
                 } else {
                     const u32 two = c2 + (p.undirected && !p.footnote && c2 != kWalkMany ? deg : 0u);
