@@ -253,9 +253,9 @@ bcm_status bcm_topk(bcm_graph_t g, uint32_t k, const bcm_options* opt, uint32_t*
  * to its own stream, so runs on different graphs overlap on the device).
  * bcm_topk_start takes bcm_topk's arguments, enqueues the run and the copies
  * of its results on the graph's stream and returns without waiting.  The
- * output arrays must stay valid until the run is finished; for the host
- * copies to be asynchronous they must be pinned host memory (pageable
- * memory works, but the copy then blocks the calling thread).  If the graph
+ * output arrays must stay valid until the run is finished: host arrays are
+ * filled by bcm_topk_finish (the copies off the device go to pinned memory of
+ * the library's own), device arrays (BCM_OUT_DEVICE) by the run itself.  If the graph
  * has not been preprocessed yet, that happens first, synchronously.
  * bcm_topk_finish(wait = 1) waits for the run and returns its outcome, as
  * bcm_topk would, filling stats (may be NULL); with wait = 0 it returns

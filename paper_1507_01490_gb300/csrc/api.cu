@@ -263,20 +263,30 @@ struct RunRes {                 // per-graph CUDA objects, reused across graphs
 };
 static std::vector<RunRes> g_res_free;
 
-// Small per-run state of the wave kernels (all zeroed before a run).
-struct Aux {
+// What a run leaves for the host, the same on both sides, so that one copy
+// brings it over (eight small ones, three of them to pageable memory, were a
+// quarter of the smallest call: top-10 of BA 2000 138 -> 108 us).
+struct RunCounters {
+    int err;
+    uint32_t topk_count;
+    uint32_t trace_n;
+    uint32_t pad;
+    unsigned long long stats[ST_COUNT];        // per-CTA wave kernel
+    unsigned long long seed_stats[ST_COUNT];   // grid-wide waves, seed wave, plain kernel, all pairs
+};
+struct RunOut : RunCounters {
     uint32_t topk_id[1024];
     u64 topk_f[1024];
     uint32_t topk_r[1024];
-    uint32_t topk_count;
+};
+
+// Small per-run state of the wave kernels (all zeroed before a run).
+struct Aux : RunOut {
     uint32_t lock;
     uint32_t head;
-    int err;
     Threshold thr;
     Threshold ext;        // key offered by bcm_topk_offer (written by the host while the run goes on)
     Threshold snap;       // the threshold all blocks of a grid-wide or plain launch cut with
-    unsigned long long stats[ST_COUNT];        // per-CTA wave kernel
-    unsigned long long seed_stats[ST_COUNT];   // seed wave / plain kernel
     GridBarrier bar;
     uint32_t gcnt[2 * kCntParity];
     uint32_t glist_n[2];
@@ -285,7 +295,6 @@ struct Aux {
     unsigned long long garc[2];
     HeavyEntry gheavy[2048];
     uint32_t gheavy_n;
-    uint32_t trace_n;
     uint32_t defer_n;     // sources handed back by per-CTA waves
     uint32_t head2;       // queue head of the grid-wide pass over them
     uint32_t walk_left[2];   // sources left by the prefilter, and by the second one
@@ -298,15 +307,11 @@ struct Aux {
     uint32_t light;       // a narrow grid-wide wave has ended the grid phase
 };
 
-// Host side of a run in flight: pinned memory the run's counters are copied
-// into, read once the run's last event has completed.
-struct HostBlock {
-    int err;
-    uint32_t topk_count;
-    uint32_t trace_n;
+// Host side of a run in flight: pinned memory the run's counters (and the
+// top-k, where its outputs are host memory) are copied into, read once the
+// run's last event has completed.
+struct HostBlock : RunOut {
     int not_simple;            // preprocessing: the simple-graph check
-    unsigned long long stats[ST_COUNT];        // per-CTA wave kernel
-    unsigned long long seed_stats[ST_COUNT];   // grid-wide or plain kernel
     // bcm_topk_threshold / bcm_topk_offer staging (helper stream)
     u64 rd_seq[2];
     Threshold rd;
@@ -363,6 +368,9 @@ struct bcm_graph {
         bool sparse = false;      // the per-CTA phase ran one source per CTA
         int lat = 0;              // ... on the padded adjacency of this many entries per row
         uint32_t kk = 0;          // entries the top-k must hold
+        uint32_t* ids = nullptr;  // host outputs of a top-k run, filled when it is finished
+        uint64_t* far = nullptr;
+        uint32_t* reach = nullptr;
         uint32_t flags = 0;
         uint64_t l0 = 0;          // launch counter at the start
         double pms = 0;           // preprocessing time of this call
@@ -1246,16 +1254,17 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     }
     Aux* a = g->d_aux;
     HostBlock* h = g->h;
-    CU(cudaMemcpyAsync(&h->err, &a->err, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
-    CU(cudaMemcpyAsync(&h->topk_count, &a->topk_count, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "copy");
-    CU(cudaMemcpyAsync(&h->trace_n, &a->trace_n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "copy");
-    CU(cudaMemcpyAsync(h->stats, a->stats, sizeof(h->stats), cudaMemcpyDeviceToHost, s), "copy");
-    CU(cudaMemcpyAsync(h->seed_stats, a->seed_stats, sizeof(h->seed_stats), cudaMemcpyDeviceToHost, s), "copy");
     const bool dev = (c.flags & BCM_OUT_DEVICE) != 0;
+    const bool host_topk = !exhaustive && !dev;
+    CU(cudaMemcpyAsync((RunCounters*)h, (RunCounters*)a, host_topk ? sizeof(RunOut) : sizeof(RunCounters),
+                       cudaMemcpyDeviceToHost, s), "copy");
+    g->pend.ids = host_topk ? (uint32_t*)o_ids : nullptr;
+    g->pend.far = host_topk ? (uint64_t*)o_far : nullptr;
+    g->pend.reach = host_topk ? (uint32_t*)o_reach : nullptr;
     if (exhaustive) {
         if ((st = copy_out(o_far, g->d_far, (size_t)g->n * sizeof(uint64_t), dev, s))) return st;
         if ((st = copy_out(o_reach, g->d_reach, (size_t)g->n * sizeof(uint32_t), dev, s))) return st;
-    } else {
+    } else if (dev) {
         const uint32_t kk = k < n_src ? k : n_src;
         if ((st = copy_out(o_ids, a->topk_id, kk * sizeof(uint32_t), dev, s))) return st;
         if ((st = copy_out(o_far, a->topk_f, kk * sizeof(uint64_t), dev, s))) return st;
@@ -1315,6 +1324,11 @@ bcm_status finish_run(bcm_graph* g, bool wait, unsigned long long* sv, unsigned 
         // a timed-out run may leave words set: do not reuse the region
         region_release(g->slots, false);
         return check_dev_err(h->err);
+    }
+    if (g->pend.ids) {
+        memcpy(g->pend.ids, h->topk_id, g->pend.kk * sizeof(uint32_t));
+        memcpy(g->pend.far, h->topk_f, g->pend.kk * sizeof(uint64_t));
+        memcpy(g->pend.reach, h->topk_r, g->pend.kk * sizeof(uint32_t));
     }
     // with an offered key a shard keeps only sources that rank before it: fewer entries are fine
     if (!g->pend.exhaustive && (offered ? h->topk_count > g->pend.kk : h->topk_count != g->pend.kk))
@@ -1554,6 +1568,7 @@ bcm_status bcm_topk_start(bcm_graph_t g, uint32_t k, const bcm_options* opt, uin
         g->pend.sparse = false;
         g->pend.lat = 0;
         g->pend.kk = 0;
+        g->pend.ids = nullptr;
         g->pend.flags = 0;
     }
     g->pend.l0 = l0;
