@@ -16,8 +16,9 @@
 // bytes per cluster: C is chosen so that those of all clusters fit in L2
 // together and no SM is idle.
 //
-// What bounds it: the gathers of F (one L2 sector per arc and level until x has
-// all lanes): about one per clock and SM.  farness of every vertex, grid-wide
+// What bounds it: the latency of the gathers of F (one L2 sector per arc and
+// level until x has all lanes; Chung-Lu 2^14: long-scoreboard stalls 16 of 28
+// cycles per issue, L1 60% busy, issue 24%): farness of every vertex, grid-wide
 // kernel -> here: Chung-Lu 2^14 36.6 -> 0.74 ms, R-MAT 2^16 103 -> 12.5; without
 // allocation (in-arcs unknown, level 1 pulled) Chung-Lu 10,007 5.3 -> 0.6 ms.
 #include <cuda_runtime.h>
