@@ -334,7 +334,8 @@ bcm_status bcm_trace(bcm_graph_t g, uint64_t* records, uint32_t cap, uint32_t* c
  * bcm_graph_trim -- give back the graph's run workspace (wave-kernel slots,
  * exhaustive outputs, plain-run buffers, trace): the slots go to a cache of
  * clean regions that other graphs' runs reuse, the rest is freed.  The CSR
- * and the preprocessing results stay.  The next run allocates again.
+ * and the preprocessing results stay, and so do the buffers that a batch of
+ * this graph uses.  The next run allocates again.
  */
 bcm_status bcm_graph_trim(bcm_graph_t g);
 
@@ -385,7 +386,10 @@ bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uint32_t* col,
  * reach[i] given at creation (they must stay valid).  Only graphs below the
  * grid-wide threshold (n * grid_lanes/64 < heavy_words) can be batched: their
  * runs hold no cooperative launch.  A graph of a batch must not run anything
- * else while a batch run is in flight.  Errors: BCM_ERR_INVALID,
+ * else while a batch run is in flight; between batch runs it may run anything,
+ * with any options: the batch keeps workspaces of its own, and the buffers it
+ * shares with its graphs stay until it is destroyed (bcm_graph_trim keeps
+ * them).  The graphs must outlive the batch's last run.  Errors: BCM_ERR_INVALID,
  * BCM_ERR_UNSUPPORTED (a graph too large, or plain / traced / grid-only /
  * sharded options), BCM_ERR_OOM, BCM_ERR_CUDA, BCM_ERR_TIMEOUT.
  */

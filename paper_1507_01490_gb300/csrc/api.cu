@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -359,6 +360,8 @@ struct bcm_graph {
     uint32_t* d_reach = nullptr;
     uint32_t* d_rank = nullptr;            // [n] all pairs, top-k runs: vertices that rank before
     Region slots{0, nullptr, 0, Layout{}};
+    std::shared_ptr<int> pin;      // shared with every batch this graph is in: bcm_graph_trim then keeps the buffers
+                                   // that recorded runs use
     int sms = 0;
     // the run started by bcm_topk_start (or a synchronous call) until finished
     struct Pending {
@@ -996,9 +999,11 @@ Walks carve_walks(bcm_graph* g) {
 // Enqueues one run of the wave kernels on the graph's stream and the copies
 // of its results and counters, and returns without waiting.  exhaustive:
 // every source, no cut, outputs o_far/o_reach (n entries); else top-k with
-// outputs o_ids/o_far/o_reach (min(k, n) entries).
+// outputs o_ids/o_far/o_reach (min(k, n) entries).  recording: the run is
+// captured, not executed; it takes the paths whose buffers the run before the
+// capture left, and lays nothing out.
 bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, void* o_ids, void* o_far,
-                     void* o_reach) {
+                     void* o_reach, bool recording = false) {
     cudaStream_t s = g->stream;
     const bool trace = (c.flags & BCM_TRACE) != 0;
     bcm_status st = ensure_aux(g);
@@ -1006,7 +1011,7 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
     if ((st = ensure_run_state(g, trace))) return st;
     const bool plain = !exhaustive && (c.flags & BCM_PLAIN);
     ApShape ap;
-    bool pairs = !plain && all_pairs_shape(g, c, exhaustive, k, &ap);
+    bool pairs = !plain && all_pairs_shape(g, c, exhaustive, k, &ap) && (!recording || g->rows_ready);
     if (pairs && !g->d_rows && buf_get_t(&g->d_rows, sorted_rows_bytes(g->n, g->m)) != cudaSuccess) {
         cudaGetLastError();   // no room for its rows: the wave kernels need none
         g->d_rows = nullptr;
@@ -1128,7 +1133,8 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         // walks alone as soon as a threshold exists -- after the first grid
         // waves, or the seed wave -- and only the others are searched
         bool filter = g->simple && !exhaustive && !c.sparse &&
-                      !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY));
+                      !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY)) &&
+                      (!recording || (g->d_surv && g->walks_base));
         if (filter && !g->d_surv && buf_get_t(&g->d_surv, walks_bytes(g->n)) != cudaSuccess) {
             cudaGetLastError();   // no room: the waves do without
             g->d_surv = nullptr;
@@ -1200,7 +1206,7 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         }
         pc.stats = g->d_aux->stats;
         cudaEventRecord(g->ev[1], s);
-        bool landmarks = c.landmarks && !exhaustive;
+        bool landmarks = c.landmarks && !exhaustive && (!recording || g->d_lm);
         if (landmarks && !g->d_lm && buf_get_t(&g->d_lm, landmark_bytes(g->n)) != cudaSuccess) {
             cudaGetLastError();   // no room: the searches do without
             g->d_lm = nullptr;
@@ -1710,19 +1716,21 @@ bcm_status bcm_graph_trim(bcm_graph_t g) {
     if (g->pend.active) return fail(BCM_ERR_INVALID, "a run on this graph has not been finished");
     CU(g->stream ? cudaStreamSynchronize(g->stream) : cudaDeviceSynchronize(), "synchronize");
     region_release(g->slots, true);
-    for (void* b : {(void*)g->d_plain, (void*)g->d_far, (void*)g->d_reach, (void*)g->d_trace, (void*)g->d_defer,
-                    (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lm, (void*)g->d_rank})
+    for (void* b : {(void*)g->d_plain, (void*)g->d_trace, (void*)g->d_shard}) buf_put(b);
+    g->d_plain = nullptr;
+    g->d_trace = nullptr;
+    g->d_shard = nullptr;
+    g->trace_n = 0;
+    if (g->pin.use_count() > 1) return BCM_OK;   // a batch's recorded runs use the others
+    for (void* b : {(void*)g->d_far, (void*)g->d_reach, (void*)g->d_defer, (void*)g->d_surv, (void*)g->d_lm,
+                    (void*)g->d_rank})
         buf_put(b);
     g->d_rank = nullptr;
     g->d_lm = nullptr;
     g->d_surv = nullptr;
     g->d_defer = nullptr;
-    g->d_shard = nullptr;
-    g->d_plain = nullptr;
     g->d_far = nullptr;
     g->d_reach = nullptr;
-    g->d_trace = nullptr;
-    g->trace_n = 0;
     return BCM_OK;
 }
 
@@ -1777,6 +1785,13 @@ struct bcm_batch {
     cudaStream_t stream = nullptr;
     std::vector<bcm_graph*> graphs;
     std::vector<uint32_t> kk;     // entries each run must hold
+    // the slot regions whose addresses are recorded, taken from the handles: a
+    // run on a handle by itself acquires another, so neither sees what the
+    // other left there, and none is released while a replay may write to it
+    std::vector<Region> regions;
+    std::vector<std::shared_ptr<int>> pins;   // the handles' other buffers stay too (bcm_graph_trim)
+    bool unclean = false;         // a replay failed: the regions are cleared before the next one
+    bool unchecked = false;       // ... may have: it was not waited for
 };
 
 static bcm_status batch_fail(bcm_batch* b, bcm_status st) {
@@ -1802,7 +1817,19 @@ bcm_status bcm_batch_create(bcm_graph_t* graphs, uint32_t count, const uint32_t*
     bcm_batch* b = new (std::nothrow) bcm_batch();
     if (!b) return fail(BCM_ERR_OOM, "host allocation");
     b->stream = (cudaStream_t)stream;
-    std::vector<Cfg> cfg(count);
+    std::vector<Cfg> cfg;
+    try {
+        cfg.resize(count);
+        b->graphs.reserve(count);
+        b->kk.reserve(count);
+        b->regions.reserve(count);
+        b->pins.reserve(count);
+        for (uint32_t i = 0; i < count; ++i)
+            if (graphs[i] && !graphs[i]->pin) graphs[i]->pin = std::make_shared<int>(0);
+    } catch (...) {
+        fail(BCM_ERR_OOM, "host allocation");
+        return batch_fail(b, BCM_ERR_OOM);
+    }
     // every run once, outside the capture: preprocessing, workspaces and
     // buffers are allocated here, and each run is checked
     for (uint32_t i = 0; i < count; ++i) {
@@ -1866,7 +1893,7 @@ bcm_status bcm_batch_create(bcm_graph_t* graphs, uint32_t count, const uint32_t*
         bcm_graph* g = graphs[i];
         cudaStream_t keep = g->stream;
         g->stream = br[i % nbr];
-        st = start_run(g, cfg[i], k[i], false, ids[i], farness[i], reach[i]);
+        st = start_run(g, cfg[i], k[i], false, ids[i], farness[i], reach[i], true);
         g->pend.active = false;   // recorded, not running
         g->stream = keep;
     }
@@ -1889,6 +1916,13 @@ bcm_status bcm_batch_create(bcm_graph_t* graphs, uint32_t count, const uint32_t*
     for (auto x : ev)
         if (x) cudaEventDestroy(x);
     if (st) return batch_fail(b, st);
+    for (uint32_t i = 0; i < count; ++i) {
+        bcm_graph* g = graphs[i];
+        b->pins.push_back(g->pin);
+        if (!g->slots.ptr) continue;   // (a graph given twice: taken already)
+        b->regions.push_back(g->slots);
+        g->slots = Region{0, nullptr, 0, Layout{}};
+    }
     *out = b;
     return BCM_OK;
 }
@@ -1896,13 +1930,19 @@ bcm_status bcm_batch_create(bcm_graph_t* graphs, uint32_t count, const uint32_t*
 bcm_status bcm_batch_run(bcm_batch_t b, int wait) {
     t_err.clear();
     if (!b) return fail(BCM_ERR_INVALID, "batch is NULL");
+    if (b->unclean) {
+        for (const Region& r : b->regions) CU(cudaMemsetAsync(r.ptr, 0, r.bytes, b->stream), "workspace clear");
+        b->unclean = false;
+    }
+    b->unchecked = true;
     CU(cudaGraphLaunch(b->exec, b->stream), "graph launch");
     if (!wait) return BCM_OK;
     CU(cudaStreamSynchronize(b->stream), "batch run");
+    b->unchecked = false;
     for (size_t i = 0; i < b->graphs.size(); ++i) {
         const HostBlock* h = b->graphs[i]->h;
         if (h->err) {
-            region_release(b->graphs[i]->slots, false);
+            b->unclean = true;   // a timed-out run may leave words set
             bcm_status st = check_dev_err(h->err);
             return fail(st, "graph %zu of the batch: %s", i, t_err.c_str());
         }
@@ -1917,6 +1957,8 @@ bcm_status bcm_batch_destroy(bcm_batch_t b) {
     if (!b) return BCM_OK;
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->exec) cudaGraphExecDestroy(b->exec);
+    // (what is left in an all-pairs region does not matter: no layout counts on it)
+    for (Region& r : b->regions) region_release(r, r.layout.kind == 3 || !(b->unclean || b->unchecked));
     delete b;
     return BCM_OK;
 }
