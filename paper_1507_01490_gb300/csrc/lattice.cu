@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
     extern __shared__ __align__(16) u32 s_dyn[];
     __shared__ u32 s_qn[3], s_ds[3];     // per level, rotating: queue length; its vertices' degree sum
     __shared__ long long s_cut[2];       // per level parity: the f~ that stops the source
-    __shared__ u32 s_base, s_stop, s_ovf, s_skip, s_lo, s_hi;
+    __shared__ u32 s_base, s_stop, s_skip, s_lo, s_hi;
     __shared__ unsigned long long s_st[ST_COUNT];   // ctl's counters
     __shared__ ThrCache s_thr;                      // ctl's last snapshot of the threshold
     const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -162,7 +162,6 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
             sq[0] = v;
             s_qn[0] = 1; s_qn[1] = 0;
             s_ds[0] = deg; s_ds[1] = 0;
-            s_ovf = 0;
             s_lo = s_hi = v >> 5;
         }
         __syncthreads();
@@ -179,7 +178,9 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
                 nd += cnt;
                 f += (u64)d * cnt;
             }
-            if (cnt > kLatQueue && s_ovf) { end = 3; break; }
+            // (the count itself, final since the barrier, says whether the
+            // queue overflowed: every thread leaves at the same level)
+            if (cnt > p.sparse_qcap) { end = 3; break; }
             if (ctl && p.trace_lanes) lane_level(p, v, d, f, nd, g);
             if ((long long)(f - g) + (long long)(d + 2) * ((long long)x - nd) >= s_cut[d & 1]) { end = 2; break; }
             u64 nseq = 0, neseq = 0;
@@ -238,7 +239,6 @@ __global__ void __launch_bounds__(THREADS, (RW == 4 ? kLatResident : 1024) / THR
                             k += w[j];
                         }
                     } else {
-                        if (at + total > p.sparse_qcap) s_ovf = 1;
 #pragma unroll
                         for (int j = 0; j < RW; ++j) {
                             if (w[j]) {
