@@ -31,8 +31,6 @@ constexpr int kApThreads = 1024;
 constexpr u32 kApRow = 32;       // longer rows are scanned by a warp
 constexpr u32 kApBig = 4096;     // ... by a CTA
 
-size_t allpairs_slot_bytes(uint32_t n, int W) { return al256((size_t)n * W * 24 + (size_t)n * 8); }
-
 __device__ __forceinline__ void ap_barrier(int C) {
     if (C == 1) __syncthreads();
     else asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -551,39 +549,6 @@ int launch_rank_topk(const unsigned long long* far, const uint32_t* reach, uint3
     k_emit<<<(n + 255) / 256, 256, 0, s>>>(far, reach, rank, n, T);
     note_launch(2);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-// Lanes, cluster size and cluster count for n vertices on `sms` SMs, at most
-// `budget` bytes of slots; returns the SMs it keeps busy.  Where every wave of
-// 64 targets has an SM of its own: that (a cluster's barrier and its loads
-// past L1 cost more than idle SMs: Chung-Lu 1000 and 4000, C = 1: 0.043 and
-// 0.11 ms, C = 8: 0.09 and 0.18).  Else the choice that keeps most SMs busy, of
-// those the widest lanes (an arc's word then serves more targets: R-MAT 2^16,
-// 256 lanes 12.2 ms, 128 13.9), of those the smallest clusters.
-int allpairs_shape(uint32_t n, int sms, size_t budget, int lanes, int* W, int* C, int* clusters) {
-    int best = 0;
-    const uint32_t one = (n + 63) / 64;
-    if (!lanes && one <= (uint32_t)sms && one * allpairs_slot_bytes(n, 1) <= budget) {
-        *W = *C = 1;
-        *clusters = (int)one;
-        return (int)one;
-    }
-    for (int w : {4, 2, 1}) {
-        if (lanes && lanes != 64 * w) continue;
-        const uint32_t waves = (n + 64 * w - 1) / (64 * w);
-        for (int c : {1, 2, 4, 8}) {
-            size_t k = budget / allpairs_slot_bytes(n, w);
-            if (k > (size_t)(sms / c)) k = (size_t)(sms / c);
-            if (k > waves) k = waves;
-            if ((int)k * c > best) {
-                best = (int)k * c;
-                *W = w;
-                *C = c;
-                *clusters = (int)k;
-            }
-        }
-    }
-    return best;
 }
 
 }  // namespace bcm

@@ -607,10 +607,7 @@ bool all_pairs_shape(bcm_graph* g, const Cfg& c, bool exhaustive, uint32_t k, Ap
         const uint64_t most = small || k > kApLongList ? kApTopkWordsMost : kApTopkWords;
         if (!c.ap_default || g->n > kAllPairsTopkN || (uint64_t)g->n * g->m / 64 > most) return false;
     }
-    const int busy = allpairs_shape(g->n, g->sms, kAllPairsL2, exhaustive ? c.ap_lanes : 0, &a->W, &a->C, &a->clusters);
-    // a large graph whose planes leave L2 with most SMs busy stays on the grid-wide kernel
-    const uint64_t waves = ((uint64_t)g->n + 64 * a->W - 1) / (64 * a->W);
-    return busy > 0 && (busy * 4 >= g->sms * 3 || (uint64_t)a->clusters == waves);
+    return allpairs_fits(g->n, g->sms, kAllPairsL2, exhaustive ? c.ap_lanes : 0, &a->W, &a->C, &a->clusters);
 }
 size_t ap_bytes(bcm_graph* g, const ApShape& a) {
     const size_t b = (size_t)a.clusters * (allpairs_slot_bytes(g->n, a.W) + kApLanesBytes);

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "shape.h"
 
 namespace bcm {
 
@@ -53,7 +54,6 @@ constexpr size_t slot_bytes(uint32_t n, int W) {
 // One-source-per-CTA slot (k_sparse): a visited bitmap of one bit per vertex,
 // the log of its words that became non-zero, then two queues of qcap
 // entries each (a frontier vertex's first arc and degree, 8 bytes).
-__host__ __device__ constexpr size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 __host__ __device__ constexpr size_t sparse_bitmap_bytes(uint32_t n) { return al256(((size_t)n + 31) / 32 * sizeof(uint32_t)); }
 __host__ __device__ constexpr size_t sparse_slot_bytes(uint32_t n, uint32_t qcap) {
     return 2 * sparse_bitmap_bytes(n) + 2 * al256((size_t)qcap * 2 * sizeof(uint32_t));
@@ -276,8 +276,6 @@ struct AllPairs {
 };
 constexpr size_t kAllPairsL2 = 130ull << 20;   // (R-MAT 2^16: 129 MB at 256 lanes 12.2 ms, 70 MB at 128 13.9)
 constexpr uint32_t kAllPairsTopkN = 16384;
-size_t allpairs_slot_bytes(uint32_t n, int W);
-int allpairs_shape(uint32_t n, int sms, size_t budget, int lanes, int* W, int* C, int* clusters);
 size_t sorted_rows_bytes(uint32_t n, uint64_t m);
 size_t sorted_rows_scratch_bytes(uint32_t n);
 int launch_sorted_rows(const uint32_t* grp, const uint32_t* gcol, const uint32_t* order, uint32_t n, uint64_t m,

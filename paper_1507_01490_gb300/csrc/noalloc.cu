@@ -135,9 +135,7 @@ extern "C" bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uin
         const bool sorted = n >= 8192 && off + rows + lane_bytes + al256(degree_order_scratch_bytes(n)) <= kNoAllocBytes / 2;
         const size_t used = off + lane_bytes + (sorted ? rows : 0);
         int W = 0, C = 0, clusters = 0;
-        const int busy = used < kNoAllocBytes ? allpairs_shape(n, sms, kNoAllocBytes - used, 0, &W, &C, &clusters) : 0;
-        const uint64_t waves = W ? ((uint64_t)n + 64 * W - 1) / (64 * W) : 0;
-        if (busy > 0 && (busy * 4 >= sms * 3 || (uint64_t)clusters == waves)) {
+        if (used < kNoAllocBytes && allpairs_fits(n, sms, kNoAllocBytes - used, 0, &W, &C, &clusters)) {
             if (cudaMemsetAsync(hdr, 0, sizeof(NoAllocHeader), s) != cudaSuccess)
                 return noalloc_fail(BCM_ERR_CUDA, "clearing the working array failed");
             if (launch_validate(row_ptr, col, n, m, &hdr->csr_err, s) || launch_narrow_offsets(row_ptr, rp32, n, s))
