@@ -506,11 +506,10 @@ __global__ void k_emit(const unsigned long long* far, const u32* reach, const u3
     }
     if (r + 1 == (T.k < n ? T.k : n)) {
         *T.count = r + 1;
-        if (r + 1 == T.k) {   // the k-th key, as bcm_topk_threshold reads it
-            score_key(far[v], reach[v], T.thr->N, T.thr->F);
-            T.thr->id = v;
-            T.thr->valid = 1;
-            T.thr->seq = 2;
+        if (r + 1 == T.k) {   // the k-th key: bcm_topk_threshold may read it meanwhile
+            u64 N, F;
+            score_key(far[v], reach[v], N, F);
+            threshold_publish(T.thr, N, F, v);
         }
     }
 }

@@ -201,18 +201,22 @@ __device__ inline void topk_insert_locked(const TopK& T, u32 v, u64 f, u32 r) {
     vstore(T.count, cnt + 1);
 }
 
+// Writes a key under its record's sequence count.  One writer at a time.
+__device__ __forceinline__ void threshold_publish(Threshold* t, u64 N, u64 F, u32 id) {
+    atomicAdd(&t->seq, 1ull);          // odd: write in progress
+    __threadfence();
+    vstore(&t->N, N); vstore(&t->F, F); vstore(&t->id, id); vstore(&t->valid, 1u);
+    __threadfence();
+    atomicAdd(&t->seq, 1ull);          // even: consistent
+}
+
 // Publishes the k-th key (caller holds the lock).
 __device__ inline void topk_publish_locked(const TopK& T) {
     u32 cnt = vload(T.count);
     if (cnt < T.k) return;
     u64 N, F;
     score_key(vload(&T.f[T.k - 1]), vload(&T.r[T.k - 1]), N, F);
-    u32 id = vload(&T.id[T.k - 1]);
-    atomicAdd(&T.thr->seq, 1ull);          // odd: write in progress
-    __threadfence();
-    vstore(&T.thr->N, N); vstore(&T.thr->F, F); vstore(&T.thr->id, id); vstore(&T.thr->valid, 1u);
-    __threadfence();
-    atomicAdd(&T.thr->seq, 1ull);          // even: consistent
+    threshold_publish(T.thr, N, F, vload(&T.id[T.k - 1]));
 }
 
 // --------------------------------------------------------- grid barrier
