@@ -332,7 +332,8 @@ bcm_status bcm_trace(bcm_graph_t g, uint64_t* records, uint32_t cap, uint32_t* c
 
 /*
  * bcm_graph_trim -- give back the graph's run workspace (wave-kernel slots,
- * exhaustive outputs, plain-run buffers, trace): the slots go to a cache of
+ * exhaustive outputs, plain-run buffers, trace, the copies of the rows and the
+ * walk counts that runs lay out for themselves): the slots go to a cache of
  * clean regions that other graphs' runs reuse, the rest is freed.  The CSR
  * and the preprocessing results stay, and so do the buffers that a batch of
  * this graph uses.  The next run allocates again.

@@ -338,7 +338,8 @@ struct bcm_graph {
     uint32_t* d_order = nullptr;
     uint32_t* d_xlo = nullptr;
     uint32_t* d_xhi = nullptr;
-    uint32_t* d_walk = nullptr;    // [2][n] degrees, and walks of two arcs that do not turn back (the prefilter's)
+    uint32_t* d_walk = nullptr;    // [2][n] degrees, and walks of two arcs that do not turn back: the prefilter's,
+                                   // made by the first top-k run that wants them
     uint32_t* d_comp = nullptr;    // component / SCC label, smallest-member order
     uint32_t* d_rrp = nullptr;     // directed: in-arcs CSR
     uint32_t* d_rcol = nullptr;
@@ -653,6 +654,16 @@ double ms_since(std::chrono::steady_clock::time_point t0) {
     return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }
 
+// Memory of the walk counts; false where there is none (a run does without).
+size_t walk_counts_bytes(uint32_t n) { return 2 * al256((size_t)n * sizeof(uint32_t)); }
+bool ensure_walk_counts(bcm_graph* g) {
+    if (g->d_walk) return true;
+    if (buf_get_t(&g->d_walk, walk_counts_bytes(g->n)) == cudaSuccess) return true;
+    cudaGetLastError();
+    g->d_walk = nullptr;
+    return false;
+}
+
 // ------------------------------------------------------ preprocessing
 bcm_status ensure_run_state(bcm_graph* g, bool trace);
 
@@ -673,11 +684,10 @@ bcm_status preprocess(bcm_graph* g, double* ms, bool topk = false) {
         if (sc > scratch) scratch = sc;
     }
     if (!g->d_order) {
-        CU(buf_get_t(&g->d_order, nb * 6), "preprocess allocation");
+        CU(buf_get_t(&g->d_order, nb * 4), "preprocess allocation");
         g->d_xlo = (uint32_t*)((char*)g->d_order + nb);
         g->d_xhi = (uint32_t*)((char*)g->d_order + 2 * nb);
         g->d_comp = (uint32_t*)((char*)g->d_order + 3 * nb);
-        g->d_walk = (uint32_t*)((char*)g->d_order + 4 * nb);
     }
     char* d_scr = nullptr;
     CU(buf_get_t(&d_scr, scratch), "preprocess scratch");
@@ -713,14 +723,14 @@ bcm_status preprocess(bcm_graph* g, double* ms, bool topk = false) {
         }
         // the prefilter's counts: beside the components on the helper stream,
         // but after them where those take fewer launches than the degree order
+        // (a run that finds them missing makes them; lattices and the smallest
+        // graphs hardly ever want them)
+        const bool walks = topk && n >= 9728 && (g->directed || g->max_deg > kSparseMaxDeg) && ensure_walk_counts(g);
         Walks K{};
         K.c[1] = g->d_walk;
         K.c[2] = (uint32_t*)((char*)g->d_walk + nb);
         K.heavy_n = (uint32_t*)(d_simple + 16);
         K.heavy = (uint32_t*)(d_scr2 + dos + scs + 256);
-        // (a run that finds them missing makes them; lattices and the smallest
-        // graphs hardly ever want them)
-        const bool walks = topk && n >= 9728 && (g->directed || g->max_deg > kSparseMaxDeg);
         const bool walks_after = !g->directed && n <= 65536;
         g->walks_base = walks;
         if (walks && !walks_after && launch_walk_base(g->d_rp, g->d_col, n, K, !g->directed, g->aux)) {
@@ -1132,6 +1142,7 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         bool filter = g->simple && !exhaustive && !c.sparse &&
                       !(c.flags & (BCM_NO_PREFILTER | BCM_GRID_ONLY | BCM_NO_CUT | BCM_CTA_ONLY)) &&
                       (!recording || (g->d_surv && g->walks_base));
+        filter = filter && ensure_walk_counts(g);
         if (filter && !g->d_surv && buf_get_t(&g->d_surv, walks_bytes(g->n)) != cudaSuccess) {
             cudaGetLastError();   // no room: the waves do without
             g->d_surv = nullptr;
@@ -1488,7 +1499,7 @@ bcm_status bcm_graph_destroy(bcm_graph_t g) {
     for (void* b : {(void*)g->d_rp, (void*)g->d_col, (void*)g->d_order, (void*)g->d_aux, (void*)g->d_plain,
                     (void*)g->d_far, (void*)g->d_reach, (void*)g->d_rrp, (void*)g->d_rcol, (void*)g->d_trace,
                     (void*)g->d_defer, (void*)g->d_shard, (void*)g->d_surv, (void*)g->d_lat, (void*)g->d_lm, (void*)g->d_rank,
-                    (void*)g->d_rows})
+                    (void*)g->d_rows, (void*)g->d_walk})
         buf_put(b);
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -1720,8 +1731,12 @@ bcm_status bcm_graph_trim(bcm_graph_t g) {
     g->trace_n = 0;
     if (g->pin.use_count() > 1) return BCM_OK;   // a batch's recorded runs use the others
     for (void* b : {(void*)g->d_far, (void*)g->d_reach, (void*)g->d_defer, (void*)g->d_surv, (void*)g->d_lm,
-                    (void*)g->d_rank})
+                    (void*)g->d_rank, (void*)g->d_rows, (void*)g->d_lat, (void*)g->d_walk})
         buf_put(b);
+    g->d_rows = nullptr;
+    g->d_lat = nullptr;
+    g->d_walk = nullptr;
+    g->rows_ready = g->lat_ready = g->walks_base = false;
     g->d_rank = nullptr;
     g->d_lm = nullptr;
     g->d_surv = nullptr;
@@ -1972,7 +1987,7 @@ uint64_t bcm_workspace_bytes(bcm_graph_t g, const bcm_options* opt) {
         const size_t b = ap_bytes(g, ap) + (size_t)g->n * 16 + sorted_rows_bytes(g->n, g->m);
         region = b > region ? b : region;
     }
-    return (uint64_t)region + sizeof(Aux) + (uint64_t)g->n * (8 + 4 * c.lat) + walks_bytes(g->n) +
+    return (uint64_t)region + sizeof(Aux) + (uint64_t)g->n * (8 + 4 * c.lat) + walks_bytes(g->n) + walk_counts_bytes(g->n) +
            (c.landmarks ? landmark_bytes(g->n) : 0);
 }
 
