@@ -70,32 +70,59 @@ __device__ __forceinline__ bool heavy_claim(SccHeavy* H, uint32_t c, uint32_t de
 // thousands of arcs, so such rows go to a list whose arcs the whole grid
 // shares in a second kernel.  A full list leaves the row with its warp.
 constexpr uint32_t kRowHeavyCap = 4096;
+constexpr uint32_t kRowPart = 4096;
 struct RowHeavy {
-    uint32_t n;
+    unsigned long long n;              // rows << 40 | parts of all of them
     uint32_t item[kRowHeavyCap];
+    uint32_t first[kRowHeavyCap];      // the row's first part: rising, since both counts rise together
 };
+
+__device__ __forceinline__ uint32_t row_parts(uint32_t deg) { return (deg - 1) / kRowPart + 1; }
 
 __device__ __forceinline__ bool row_claim(RowHeavy* H, uint32_t u, uint32_t deg) {
     if (!H || deg <= kHeavyEdges) return false;
     uint32_t slot = 0;
-    if ((threadIdx.x & 31) == 0) slot = atomicAdd(&H->n, 1u);
+    if ((threadIdx.x & 31) == 0) {
+        const unsigned long long at = atomicAdd(&H->n, (1ull << 40) | row_parts(deg));
+        slot = (uint32_t)(at >> 40);
+        if (slot < kRowHeavyCap) {
+            H->item[slot] = u;
+            H->first[slot] = (uint32_t)at;
+        }
+    }
     slot = __shfl_sync(0xffffffffu, slot, 0);
-    if (slot >= kRowHeavyCap) return false;
-    if ((threadIdx.x & 31) == 0) H->item[slot] = u;
-    return true;
+    return slot < kRowHeavyCap;
 }
 
-// The heavy rows' arcs: each row is shared by kRowParts blocks, the rows by the
-// grid (row after row over the whole grid, one step each, took a load's latency
-// per row: 0.3 to 0.6 ms a pass on R-MAT 2^20's few hundred heavy rows).
-// bcm_scc_bounds of R-MAT 2^18: 2.15 -> 1.86 ms.
-constexpr uint32_t kRowParts = 4;
-#define ROW_HEAVY_LOOP(H, rp, u, e)                                                                        \
-    const uint32_t hn_ = ((H)->n < kRowHeavyCap ? (H)->n : kRowHeavyCap) * kRowParts;                     \
-    for (uint32_t h_ = blockIdx.x; h_ < hn_; h_ += gridDim.x)                                              \
-        for (uint32_t u = (H)->item[h_ / kRowParts], e_end_ = (rp)[u + 1],                                 \
-                      e = (rp)[u] + (h_ % kRowParts) * blockDim.x + threadIdx.x;                           \
-             e < e_end_ && e >= (rp)[u]; e += kRowParts * blockDim.x)
+// Part t of the listed rows, kRowPart arcs of one row; a block takes t =
+// blockIdx.x, blockIdx.x + gridDim.x, ...: a row of 10^4 arcs gets a few blocks,
+// one of 10^6 hundreds.  (The whole grid on row after row took a load's latency
+// per row, 0.3 to 0.6 ms a pass on R-MAT 2^20's few hundred; four blocks a row
+// whatever its length took a row of 10^6 arcs in a thousand dependent steps.
+// bcm_scc_bounds, the three ways: R-MAT 2^18 2.02, 1.72 and 1.72 ms, 2^20 3.85,
+// 2.78 and 2.73; 1.2 M vertices, one row of 10^6 arcs 2.80, 3.97 and 2.84.  Parts
+// of 2,048 or 8,192 arcs: within 1%.)
+// The row is found by the warp, 32 of the rising `first` a round, three at most.
+struct RowPart { uint32_t u, beg, end; };
+__device__ __forceinline__ bool row_part(const RowHeavy* H, const uint32_t* rp, uint32_t t, RowPart& r) {
+    const unsigned long long n = H->n;
+    const uint32_t rows = (uint32_t)(n >> 40), lane = threadIdx.x & 31;
+    uint32_t lo = 0, len = rows < kRowHeavyCap ? rows : kRowHeavyCap;
+    if (len == 0) return false;
+    while (len > 1) {
+        const uint32_t step = (len + 31) / 32, i = lo + lane * step;
+        const uint32_t k = __popc(__ballot_sync(0xffffffffu, i < lo + len && H->first[i] <= t));   // (at least one: first[0] = 0)
+        const uint32_t skip = (k - 1) * step;
+        lo += skip;
+        len = len - skip < step ? len - skip : step;
+    }
+    r.u = H->item[lo];
+    const uint32_t b = rp[r.u], e = rp[r.u + 1], j = t - H->first[lo];
+    if (j >= row_parts(e - b)) return false;   // past the last listed row
+    r.beg = b + j * kRowPart;
+    r.end = e - r.beg < kRowPart ? e : r.beg + kRowPart;
+    return true;
+}
 
 __global__ void k_count_in(const uint32_t* rp, const uint32_t* col, uint32_t n, uint32_t* indeg, RowHeavy* H) {
     WARP_PER_ITEM(u, n) {
@@ -105,7 +132,9 @@ __global__ void k_count_in(const uint32_t* rp, const uint32_t* col, uint32_t n, 
 }
 
 __global__ void k_count_in_heavy(const uint32_t* rp, const uint32_t* col, uint32_t* indeg, const RowHeavy* H) {
-    ROW_HEAVY_LOOP(H, rp, u, e) atomicAdd(&indeg[col[e]], 1u);
+    RowPart r;
+    for (uint32_t t = blockIdx.x; row_part(H, rp, t, r); t += gridDim.x)
+        for (size_t e = (size_t)r.beg + threadIdx.x; e < r.end; e += blockDim.x) atomicAdd(&indeg[col[e]], 1u);
 }
 
 __global__ void k_fill_rev(const uint32_t* rp, const uint32_t* col, uint32_t n, uint32_t* cursor, uint32_t* rcol,
@@ -118,7 +147,10 @@ __global__ void k_fill_rev(const uint32_t* rp, const uint32_t* col, uint32_t n, 
 
 __global__ void k_fill_rev_heavy(const uint32_t* rp, const uint32_t* col, uint32_t* cursor, uint32_t* rcol,
                                  const RowHeavy* H) {
-    ROW_HEAVY_LOOP(H, rp, u, e) rcol[atomicAdd(&cursor[col[e]], 1u)] = u;
+    RowPart r;
+    for (uint32_t t = blockIdx.x; row_part(H, rp, t, r); t += gridDim.x)
+        for (size_t e = (size_t)r.beg + threadIdx.x; e < r.end; e += blockDim.x)
+            rcol[atomicAdd(&cursor[col[e]], 1u)] = r.u;
 }
 
 __global__ void k_set_last(uint32_t* a, uint32_t idx, uint32_t v) { a[idx] = v; }
@@ -374,18 +406,16 @@ __global__ void k_dag_keys(const uint32_t* rp, const uint32_t* col, uint32_t n, 
     ks.flush();
 }
 
-// the rows row_claim listed, shared as in ROW_HEAVY_LOOP, 32 arcs per warp at a time
+// the rows row_claim listed, part by part, 32 arcs per warp at a time
 __global__ void k_dag_keys_heavy(const uint32_t* rp, const uint32_t* col, const uint32_t* comp, int b,
                                  unsigned long long* keys, uint32_t* kcnt, const RowHeavy* H) {
     __shared__ unsigned long long s_stage[8 * kKeyStage];
     KeyStage ks{&s_stage[(threadIdx.x >> 5) * kKeyStage], keys, kcnt, 0};
-    const uint32_t hn = (H->n < kRowHeavyCap ? H->n : kRowHeavyCap) * kRowParts;
-    const uint32_t lane = threadIdx.x & 31, warps = blockDim.x / 32;
-    for (uint32_t h = blockIdx.x; h < hn; h += gridDim.x) {
-        const uint32_t u = H->item[h / kRowParts], beg = rp[u], end = rp[u + 1], cu = comp[u];
-        for (size_t e0 = beg + (size_t)((h % kRowParts) * warps + threadIdx.x / 32) * 32; e0 < end;
-             e0 += (size_t)kRowParts * warps * 32)
-            dag_key(col, comp, cu, b, (uint32_t)(e0 + lane), e0 + lane < end, ks);
+    RowPart r;
+    for (uint32_t t = blockIdx.x; row_part(H, rp, t, r); t += gridDim.x) {
+        const uint32_t cu = comp[r.u];
+        for (size_t e0 = (size_t)r.beg + (threadIdx.x & ~31u); e0 < r.end; e0 += blockDim.x)
+            dag_key(col, comp, cu, b, (uint32_t)(e0 + (threadIdx.x & 31)), e0 + (threadIdx.x & 31) < r.end, ks);
     }
     ks.flush();
 }
@@ -707,13 +737,13 @@ int launch_reverse_csr(const uint32_t* rp, const uint32_t* col, uint32_t n, uint
     if (!cursor || !total || !scan_scr || !H) return -1;
     const unsigned gw = grid_for((size_t)n * 32);
     cudaMemsetAsync(cursor, 0, ((size_t)n + 1) * 4, s);
-    cudaMemsetAsync(&H->n, 0, 4, s);
+    cudaMemsetAsync(&H->n, 0, sizeof(H->n), s);
     LAUNCH(k_count_in<<<gw, 256, 0, s>>>(rp, col, n, cursor, H));
     LAUNCH(k_count_in_heavy<<<152 * 8, 256, 0, s>>>(rp, col, cursor, H));
     if (exclusive_scan_u32(cursor, rrp, n, total, scan_scr, s)) return -1;
     LAUNCH(k_set_last<<<1, 1, 0, s>>>(rrp, n, (uint32_t)m));
     cudaMemcpyAsync(cursor, rrp, (size_t)n * 4, cudaMemcpyDeviceToDevice, s);
-    cudaMemsetAsync(&H->n, 0, 4, s);
+    cudaMemsetAsync(&H->n, 0, sizeof(H->n), s);
     LAUNCH(k_fill_rev<<<gw, 256, 0, s>>>(rp, col, n, cursor, rcol, H));
     LAUNCH(k_fill_rev_heavy<<<152 * 8, 256, 0, s>>>(rp, col, cursor, rcol, H));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -868,7 +898,7 @@ int launch_scc_bounds(const uint32_t* rp, const uint32_t* col, const uint32_t* r
         void* rscr = B.take(radix_scratch_bytes(m));
         if (!keys || !ktmp || !dsrc || !ddst || !rscr) return -1;
         RowHeavy* RH = (RowHeavy*)heavy;   // the SCC heavy area is free here and at least as large
-        cudaMemsetAsync(&RH->n, 0, 4, s);
+        cudaMemsetAsync(&RH->n, 0, sizeof(RH->n), s);
         cudaMemsetAsync(&cnts[5], 0, 4, s);
         LAUNCH(k_dag_keys<<<gw, 256, 0, s>>>(rp, col, n, comp, b, keys, &cnts[5], RH));
         LAUNCH(k_dag_keys_heavy<<<152 * 8, 256, 0, s>>>(rp, col, comp, b, keys, &cnts[5], RH));
