@@ -1,0 +1,70 @@
+"""Walk counts on graphs above 65,536 vertices, where each is a launch of its
+own: three and four arcs deep (the k-th entry is far from the others), on
+undirected graphs and digraphs, with rows for a thread, a warp, a block and a
+cluster of blocks.  Whole numbers, against the oracle's search from every
+vertex: exact.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+    from paper_1507_01490_gb300 import _build, bcm
+    _build.build_cuda()
+    bcm.load()
+    return bcm
+
+
+def _graph(gen, directed):
+    """A part of 50,000 vertices with long distances, beside stars whose centres' rows take a cluster (20,000 arcs and
+    16,385) and a block (16,384: the longest, and 1,500)."""
+    rng = np.random.default_rng(11)
+    n = 50000
+    if directed:
+        src, dst = [np.repeat(np.arange(n), 2)], [rng.integers(0, n, 2 * n)]
+    else:
+        base = gen.ba(n, 1, seed=4)
+        src, dst = [np.repeat(np.arange(n), base.degrees())], [base.col]
+    at = n
+    for arcs in (20000, 16385, 16383, 1499):   # (one more to the tail)
+        src.append(np.full(arcs, at))
+        dst.append(at + 1 + np.arange(arcs))
+        src.append(np.r_[at, at + arcs + 1 + np.arange(599)])
+        dst.append(at + arcs + 1 + np.arange(600))
+        at += arcs + 601
+    return gen.csr_from_arcs(at, np.concatenate(src), np.concatenate(dst), directed=directed, name="walks%d" % directed)
+
+
+@pytest.mark.parametrize("directed", [False, True])
+def test_three_and_four_arcs(B, gen, orc, directed):
+    g = _graph(gen, directed)
+    assert g.n > 65536
+    f, r = orc.farness_all(g)
+    for k in (1, 10, 100):
+        ids = orc.topk(f, r, k)
+        assert f[ids[-1]] > 3.75 * (r[ids[-1]] - 1)   # the distance at which counts of four arcs are taken
+        with B.BcmGraph.from_graph(g) as h:
+            for kw in ({}, {}, dict(heavy_words=1)):
+                got = h.topk(k, **kw)
+                assert np.array_equal(got[0], ids) and np.array_equal(got[1], f[ids]) and np.array_equal(got[2], r[ids]), \
+                    (k, kw)
+
+
+def test_one_hub_of_a_million(B, gen):
+    """Preprocessing of a star for a top-k run, its one long row among the walk counts': by one block 0.44 ms, by a
+    cluster 0.29; the mean of both is the bound, on the best of 20."""
+    g = gen.star(1 << 20)
+    best = np.inf
+    for _ in range(20):
+        with B.BcmGraph.from_graph(g) as h:
+            ids, far, reach, st = h.topk(1)
+        assert ids[0] == 0 and far[0] == g.n - 1 and reach[0] == g.n
+        best = min(best, st["preprocess_ms"])
+    assert best < 0.365, best
