@@ -90,14 +90,39 @@ __device__ __forceinline__ void ap_finish(u64* vis, u64* Fn, u64* acc, u32 x, u3
     }
 }
 
+// A level sweeps every row, whatever it gains, so on graphs whose searches are
+// thin (long chains, rings, many small parts) k_wave_cta is faster, which scans
+// frontiers only: without allocation, 65,536 vertices in paths of ten took 11.6
+// ms against its 2.9, a ring of 60,000 and 40 arcs each 20.9 s against 4.5.  No
+// count that is known beforehand tells such graphs apart, so there (kApPaced) the
+// first waves compare their pace with what that kernel takes for a level,
+// kRivalLevelNs and kRivalFoundNs for each (vertex, lane) pair that it reaches
+// (within a third of what it took on paths, cycles, rings and chains of 8,000 to
+// 130,000 vertices; on power-law graphs, where all pairs is 10 to 30 times
+// faster, it takes a tenth of that).  They look at levels 32, 64, 128, ... and at
+// their ends, and give up once half of the clusters have looked and the pace is
+// worse by a tenth -- by two before level 256, since frontiers that widen have
+// little at first (directed grids of 128^2 and 300^2: all pairs 5.7 and 725 ms,
+// k_wave_cta 45 and 3,140).  Where both take about the same the choice can be
+// wrong by a quarter.
+constexpr u64 kRivalLevelNs = 4000, kRivalFoundNs = 30;
+constexpr u32 kApQuit = 24;      // lanes: past [3][2W], three rotating copies of Pace::quit
+
+// kApSorted: p.vertex.  kApGiven: rows in any order.  kApPaced: either, p.pace.
+enum ApKind { kApSorted, kApGiven, kApPaced };
+
 // Rows are numbered by degree descending where the caller laid them out so
 // (p.vertex: the vertex of each row): a warp's 32 rows then have about the
 // same length, and the few long ones come first.
-template <int W, int C>
+template <int W, int C, ApKind KIND>
 __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
+    constexpr bool PACED = KIND == kApPaced;
     __shared__ u32 s_or[2 * W];          // lanes that gained a row, this CTA's part
     __shared__ unsigned long long s_acc[W];
-    __shared__ unsigned long long s_st;
+    __shared__ unsigned long long s_st, s_found;
+    // (PACED; thread 0's: when and where this wave was looked at last, what its CTA's rows had then)
+    __shared__ u64 s_look_ns, s_look_found;
+    __shared__ u32 s_look_d;
     const u32 tid = threadIdx.x, lane = tid & 31;
     const u32 rank = blockIdx.x % C, cl = blockIdx.x / C, ncl = gridDim.x / C;
     const u32 n = p.n;
@@ -114,11 +139,36 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
     // (unsorted rows: every row is scanned by a thread or, past kApRow, a warp)
     const u32 nbig = p.vertex ? rows_over(p.rp, n, kApBig) : 0;
     const u32 nwide = p.vertex ? rows_over(p.rp, n, kApRow) : n;
-    if (tid == 0) s_st = 0;
+    if (tid == 0) { s_st = 0; s_found = 0; }
     u64 mvis = 0;
     u32 levels = 0, maxlev = 0;
+    bool quit = false;
+    // level d of a wave has ended; `found`: the pairs this thread's rows have
+    auto look = [&](u32 d, u64 found) {
+        for (int o = 16; o; o >>= 1) found += __shfl_xor_sync(0xffffffffu, found, o);
+        if (lane == 0 && found) atomicAdd(&s_found, (unsigned long long)found);
+        __syncthreads();
+        if (tid == 0) {
+            atomicAdd(&p.pace->found, (unsigned long long)(s_found - s_look_found));
+            s_look_found = s_found;
+            s_found = 0;
+            if (rank == 0) {
+                const u64 now = global_ns(), dt = now - s_look_ns, dl = d - s_look_d;
+                s_look_ns = now;
+                s_look_d = d;
+                const u64 ns = atomicAdd(&p.pace->ns, (unsigned long long)dt) + dt;
+                const u64 lv = atomicAdd(&p.pace->levels, (unsigned long long)dl) + dl;
+                const u32 looks = atomicAdd(&p.pace->looks, 1u) + 1;
+                // time left in rounds of waves, this kernel's and the other's
+                const u64 mine = ns * ((waves + ncl - 1) / ncl);
+                const u64 other = (kRivalLevelNs * lv + kRivalFoundNs * vload(&p.pace->found) / W) * p.rival_rounds;
+                if (looks * 2 >= ncl && mine * 10 > other * (d < 256 ? 20 : 11)) vstore(&p.pace->quit, 1u);
+            }
+        }
+    };
     for (u32 wave = cl; wave < waves; wave += ncl) {
-        const u32 t0 = wave * 64 * W;
+        // (looked at, the first waves have to speak for all: where there are many, they are spread over the targets)
+        const u32 t0 = (PACED ? (u32)((u64)wave * p.wave_step % waves) : wave) * 64 * W;
         const u32 nt = n - t0 < 64u * W ? n - t0 : 64u * W;
         u64 alive[W];
 #pragma unroll
@@ -143,6 +193,11 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
         if (rank == 0 && tid < 3 * 2 * W) gor[tid] = 0;
         if (tid < 2 * W) s_or[tid] = 0;
         ap_barrier(C);
+        if (PACED && tid == 0) {
+            s_look_ns = global_ns();
+            s_look_found = 0;
+            s_look_d = 0;
+        }
         // level 1 by push where the in-arcs are there: the targets' few rows
             // instead of every arc of the graph (half to four fifths of all
             // the arcs a wave's pulls would scan)
@@ -210,8 +265,7 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
                 __syncthreads();
             }
             // long rows, one warp each
-            for (u32 x = nbig + gw; x < (pushed ? 0u : nwide); x += NW) {
-                if (!p.vertex && __ldg(&p.rp[x + 1]) - __ldg(&p.rp[x]) <= kApRow) continue;
+            auto wide_row = [&](u32 x) {
                 u64 v[W], pend[W], got[W];
                 ap_load<W, C>(&vis[(size_t)x * W], v);
                 const u32 b = __ldg(&p.rp[x]), e = __ldg(&p.rp[x + 1]);
@@ -253,6 +307,17 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
                     ap_finish<W>(vis, Fn, acc, x, d, C == 1 ? acc[x] : __ldcg(&acc[x]), v, pend, got, gain);
                 }
                 __syncwarp();
+            };
+            if (KIND != kApSorted && !p.vertex) {
+                // unsorted rows: a warp looks over 32 at a time (one at a time
+                // the lengths alone took 28 us a level at n = 8,000)
+                for (u32 x0 = gw * 32; x0 < (pushed ? 0u : n); x0 += NW * 32) {
+                    const u32 y = x0 + lane;
+                    u32 todo = __ballot_sync(0xffffffffu, y < n && __ldg(&p.rp[y + 1]) - __ldg(&p.rp[y]) > kApRow);
+                    for (; todo; todo &= todo - 1) wide_row(x0 + __ffs(todo) - 1);
+                }
+            } else {
+                for (u32 x = nbig + gw; x < (pushed ? 0u : nwide); x += NW) wide_row(x);
             }
             // the others, one thread each; where the rows are sorted, a warp's 32
             // rows lie interleaved (entry j of lane l at 32 j + l, padded to the
@@ -325,6 +390,7 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
                 // the next level's copy: last read two levels ago
                 if (rank == 0) gor[((par + 1) % 3) * 2 * W + tid] = 0;
             }
+            if (PACED && rank == 0 && tid == 0) gor[kApQuit + par] = vload(&p.pace->quit);
             ap_barrier(C);
             u64 live = 0;
 #pragma unroll
@@ -332,13 +398,21 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
                 alive[g] &= ((u64)__ldcg(&go[2 * g + 1]) << 32) | __ldcg(&go[2 * g]);
                 live |= alive[g];
             }
+            if (PACED) quit = __ldcg(&gor[kApQuit + par]) != 0;   // (the same for the whole cluster)
             par = (par + 1) % 3;
-            if (!live) break;
+            if (!live || quit) break;
+            if (PACED && wave < ncl && d >= 32 && !(d & (d - 1))) {
+                u64 found = 0;
+                for (u32 x = gw * 32 + lane; x < n; x += NW * 32) found += __ldcg(&acc[x]) >> 32;
+                look(d, found);
+            }
         }
+        if (quit) break;
         if (rank == 0 && tid == 0) { levels += d; maxlev = d > maxlev ? d : maxlev; }
         // this wave's share of every vertex's farness and reach, and of the
         // arcs a search per source would scan (deg(t) for each x that reaches
         // t): counts of the columns, most of which are full or empty
+        u64 found = 0;
         for (u32 x0 = gw * 32; x0 < n; x0 += NW * 32) {
             const u32 x = x0 + lane;
             u64 v[W];
@@ -347,6 +421,7 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
             if (x < n) {
                 ap_load<W, C>(&vis[(size_t)x * W], v);
                 const u64 a = C == 1 ? acc[x] : __ldcg(&acc[x]);
+                if (PACED) found += a >> 32;
                 if (a) {
                     const u32 y = p.vertex ? __ldg(&p.vertex[x]) : x;
                     atomicAdd(&p.far[y], (unsigned long long)(a & 0xffffffffull));
@@ -372,6 +447,8 @@ __global__ void __launch_bounds__(kApThreads) k_allpairs(AllPairs p) {
                 }
             }
         }
+        // (a wave to come, and most of them: else it is too late to give up)
+        if (PACED && wave + ncl < waves && (wave < ncl || wave * 4 < waves)) look(d, found);
         ap_barrier(C);
     }
     for (int o = 16; o; o >>= 1) mvis += __shfl_xor_sync(0xffffffffu, mvis, o);
@@ -515,14 +592,19 @@ __global__ void k_emit(const unsigned long long* far, const u32* reach, const u3
 }
 
 // ------------------------------------------------------------- launchers
-template <int W>
+template <int W, ApKind KIND>
 static const void* ap_kernel(int C) {
-    return C == 1 ? (const void*)k_allpairs<W, 1> : C == 2 ? (const void*)k_allpairs<W, 2>
-         : C == 4 ? (const void*)k_allpairs<W, 4> : (const void*)k_allpairs<W, 8>;
+    return C == 1 ? (const void*)k_allpairs<W, 1, KIND> : C == 2 ? (const void*)k_allpairs<W, 2, KIND>
+         : C == 4 ? (const void*)k_allpairs<W, 4, KIND> : (const void*)k_allpairs<W, 8, KIND>;
+}
+
+template <ApKind KIND>
+static const void* ap_kernel(int W, int C) {
+    return W == 1 ? ap_kernel<1, KIND>(C) : W == 2 ? ap_kernel<2, KIND>(C) : ap_kernel<4, KIND>(C);
 }
 
 int launch_allpairs(const AllPairs& p, int W, int C, int clusters, cudaStream_t s) {
-    const void* k = W == 1 ? ap_kernel<1>(C) : W == 2 ? ap_kernel<2>(C) : ap_kernel<4>(C);
+    const void* k = p.pace ? ap_kernel<kApPaced>(W, C) : p.vertex ? ap_kernel<kApSorted>(W, C) : ap_kernel<kApGiven>(W, C);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(clusters * C);
     cfg.blockDim = dim3(kApThreads);

@@ -1104,6 +1104,8 @@ bcm_status start_run(bcm_graph* g, const Cfg& c, uint32_t k, bool exhaustive, vo
         a.far = g->d_far;
         a.reach = g->d_reach;
         a.stats = p.stats;
+        a.pace = nullptr;   // (the grid-wide kernel is slower on every graph tried, deep ones too)
+        a.rival_rounds = a.wave_step = 0;
         CU(cudaMemsetAsync(g->d_far, 0, (size_t)g->n * sizeof(uint64_t), s), "output clear");
         CU(cudaMemsetAsync(g->d_reach, 0, (size_t)g->n * sizeof(uint32_t), s), "output clear");
         if (rc == 0) rc = launch_allpairs(a, ap.W, ap.C, ap.clusters, s);

@@ -273,6 +273,14 @@ struct AllPairs {
     unsigned long long* far;       // [n] zeroed
     uint32_t* reach;               // [n] zeroed
     unsigned long long* stats;     // [ST_COUNT]
+    // where another kernel can take over: what the waves have cost so far, and how many rounds of
+    // waves of 64 sources that kernel would run (NULL: there is none)
+    struct Pace {
+        unsigned long long ns, levels, found;   // of the levels looked at: time, their number, (row, lane) pairs gained
+        uint32_t looks, quit;                   // quit: given up, far and reach are not complete
+    }* pace;
+    uint32_t rival_rounds;
+    uint32_t wave_step;            // with pace: wave i takes the targets of wave i * wave_step mod the waves (coprime)
 };
 constexpr size_t kAllPairsL2 = 130ull << 20;   // (R-MAT 2^16: 129 MB at 256 lanes 12.2 ms, 70 MB at 128 13.9)
 constexpr uint32_t kAllPairsTopkN = 16384;

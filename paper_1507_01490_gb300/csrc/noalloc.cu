@@ -28,8 +28,9 @@ namespace bcm {
 
 // 64 MiB: the CSR offsets narrowed to 32 bits, then either the planes of as
 // many waves of k_allpairs as fit (and, where there is room, its sorted rows),
-// or, on graphs too large for most SMs to have one, a source order and the
-// per-CTA wave slots (44 bytes per vertex each) for as many CTAs as fit.
+// or, on graphs too large for most SMs to have one and on those whose searches
+// turn out thin, a source order and the per-CTA wave slots (44 bytes per vertex
+// each) for as many CTAs as fit.
 constexpr size_t kNoAllocBytes = 64ull << 20;
 constexpr uint32_t kNoAllocMaxN = 1250000;   // at least one CTA slot (44 bytes per vertex) fits
 
@@ -41,6 +42,7 @@ struct NoAllocHeader {
     int csr_err;
     uint32_t pad;
     unsigned long long stats[ST_COUNT];
+    AllPairs::Pace pace;
 };
 
 // Layout: header (256 bytes) | offsets u32[n+1] | order u32[n] | CTA slots.
@@ -131,8 +133,9 @@ extern "C" bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uin
         const size_t lane_bytes = al256((size_t)sms * 48 * sizeof(uint32_t));
         const size_t off = kHeaderBytes + al256(((size_t)n + 1) * 4);
         const size_t rows = al256((size_t)n * 4) + sorted_rows_bytes(n, m);
-        // (laying the rows out takes ten launches: 0.1 ms, as much as all of n = 1000)
-        const bool sorted = n >= 8192 && off + rows + lane_bytes + al256(degree_order_scratch_bytes(n)) <= kNoAllocBytes / 2;
+        // (laying the rows out takes ten launches: 0.1 ms, as much as all of n = 1000,
+        // or of 9,000 vertices with one arc or none)
+        const bool sorted = n >= 8192 && m >= 2 * (uint64_t)n && off + rows + lane_bytes + al256(degree_order_scratch_bytes(n)) <= kNoAllocBytes / 2;
         const size_t used = off + lane_bytes + (sorted ? rows : 0);
         int W = 0, C = 0, clusters = 0;
         if (used < kNoAllocBytes && allpairs_fits(n, sms, kNoAllocBytes - used, 0, &W, &C, &clusters)) {
@@ -163,6 +166,22 @@ extern "C" bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uin
             a.far = (unsigned long long*)farness;
             a.reach = reach;
             a.stats = hdr->stats;
+            // thin searches are left to the per-CTA waves below, as many at once
+            // as fit, two to an SM.  (Up to 16,384 vertices of four arcs or
+            // more, none of the graphs tried is faster there by more than 4%:
+            // a ring of 16,000 and 40 arcs each 100 ms here, 96 there, directed
+            // rings of four arcs and 8,000 and 16,000 vertices 16 and 95 here,
+            // 24 and 140 there.)
+            const bool paced = n > 16384 || m < 4 * (uint64_t)n;
+            const size_t fit = (kNoAllocBytes - noalloc_fixed_bytes(n)) / slot_bytes(n, 1);
+            const uint32_t at_once = (uint32_t)(fit < 2 * (size_t)sms ? fit : 2 * (size_t)sms);
+            a.pace = paced ? &hdr->pace : nullptr;
+            a.rival_rounds = ((n + 63) / 64 + at_once - 1) / at_once;
+            // (of two or three rounds the first speaks for the rest as it is, and
+            // any other order only packs the waves worse: paths of 16,000
+            // vertices 220 -> 267 ms)
+            const uint32_t waves = (n + 64 * W - 1) / (64 * W);
+            a.wave_step = waves > 3 * (uint32_t)clusters ? spread_step(waves) : 1;
             if (sorted) {
                 char* rbuf = (char*)order + al256((size_t)n * 4);
                 if (launch_degree_order(rp32, n, order, a.slots, degree_order_scratch_bytes(n), s) ||
@@ -174,8 +193,12 @@ extern "C" bcm_status bcm_farness_all_noalloc(const uint64_t* row_ptr, const uin
                 cudaMemsetAsync(reach, 0, (size_t)n * sizeof(uint32_t), s) != cudaSuccess)
                 return noalloc_fail(BCM_ERR_CUDA, "clearing the outputs failed");
             if (launch_allpairs(a, W, C, clusters, s)) return noalloc_fail(BCM_ERR_CUDA, "wave kernel launch failed");
+            uint32_t quit = 0;
+            if (paced && cudaMemcpyAsync(&quit, &hdr->pace.quit, sizeof(quit), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+                return noalloc_fail(BCM_ERR_CUDA, "wave kernel failed");
             if (cudaStreamSynchronize(s) != cudaSuccess) return noalloc_fail(BCM_ERR_CUDA, "wave kernel failed");
-            return BCM_OK;
+            if (!quit) return BCM_OK;
+            // thin searches: the waves below are faster, and write every output
         }
     }
     const size_t fixed = noalloc_fixed_bytes(n);

@@ -52,6 +52,16 @@ inline int allpairs_shape(uint32_t n, int sms, size_t budget, int lanes, int* W,
     return best;
 }
 
+// A number coprime to `count`, near the golden ratio of it: i * step mod count, i
+// = 0, 1, ..., visits every number once, and any first few are spread evenly.
+inline uint32_t spread_step(uint32_t count) {
+    for (uint32_t s = (uint32_t)((uint64_t)count * 618 / 1000);; ++s) {
+        uint32_t a = count, b = s;
+        while (b) { const uint32_t t = a % b; a = b; b = t; }
+        if (a == 1) return s;
+    }
+}
+
 // Is that shape worth taking?  A large graph whose planes leave L2 (`budget`)
 // with most SMs idle stays on the kernels that search from sources; so does one
 // that no shape fits.

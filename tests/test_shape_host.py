@@ -43,3 +43,20 @@ def test_every_size_gets_an_answer(tmp_path):
     assert res.returncode == 0, (res.returncode, res.stdout)   # (a division by zero ends it by a signal on x86)
     taken, left = map(int, res.stdout.split())
     assert taken > 1000 and left > 1000
+
+
+def test_spread_steps(tmp_path):
+    """i * spread_step(count) mod count visits every number below count once."""
+    src, exe = tmp_path / "step.cc", tmp_path / "step"
+    src.write_text('#include <cstdio>\n#include <vector>\n#include "shape.h"\n'
+                   'int main() {\n'
+                   '    for (uint32_t c = 1; c <= 4500; ++c) {\n'
+                   '        std::vector<char> seen(c);\n'
+                   '        const uint64_t s = bcm::spread_step(c);\n'
+                   '        for (uint32_t i = 0; i < c; ++i) if (seen[i * s % c]++) { std::printf("%u\\n", c); return 1; }\n'
+                   '    }\n'
+                   '    return 0;\n}\n')
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_1507_01490_gb300", "csrc"), str(src),
+                    "-o", str(exe)], check=True)
+    res = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert res.returncode == 0, res.stdout
