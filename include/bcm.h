@@ -103,9 +103,10 @@ typedef enum {
  * is stopped and its sources run again on the grid kernel after the
  * per-CTA phase (see defer_words).  Exhaustive runs stay on the grid
  * kernel (with BCM_SPARSE, on the one-source kernel); with no flag but
- * BCM_OUT_DEVICE / BCM_NO_FOOTNOTE they run on the all-pairs kernel (targets
- * as lanes) where its bit planes stay in L2 (up to about 130,000 vertices), and
- * top-k runs of small graphs with no launch parameter set take their answer
+ * BCM_OUT_DEVICE / BCM_NO_FOOTNOTE, no shard and no short wait_limit_ns they run
+ * on the all-pairs kernel (targets as lanes) where the bit planes of enough
+ * waves for three quarters of the SMs fit 130 MB, about L2's size (up to about
+ * 284,000 vertices), and top-k runs of small graphs with no launch parameter set take their answer
  * from every vertex's farness by that kernel (n <= 16,384 and n m below 2^30,
  * or 2^32 for k > 32 or n < 9,728).  Levels of grid waves
  * run by push (each frontier vertex
@@ -138,7 +139,9 @@ typedef struct {
                                  as many out-arcs) stops and hands its live sources to a second
                                  grid-wide pass, which runs them from the start; 0 = default
                                  (heavy_words) */
-    uint64_t wait_limit_ns;   /* limit of every in-kernel wait; 0 = default (20 s) */
+    uint64_t wait_limit_ns;   /* limit of every in-kernel wait; 0 = default (20 s).  With a limit below the
+                                 default, runs stay on the kernels that it is asked of: none on the
+                                 all-pairs kernel, which waits for nothing but its own thread blocks */
     uint32_t shard_index;     /* bcm_topk over one shard of the sources (several GPUs, one graph):  */
     uint32_t shard_count;     /* the positions p of the degree order with (p / 64) % shard_count ==
                                  shard_index; the result is that shard's own top-k, min(k, shard

@@ -475,7 +475,8 @@ bcm_status resolve(bcm_graph* g, const bcm_options* opt, Cfg* c) {
                                             g->max_deg <= kSparseMaxDeg));
     // settings as the library chooses them: all pairs where that is cheap
     c->all_pairs = !(o.flags & ~(BCM_OUT_DEVICE | BCM_NO_FOOTNOTE)) && o.shard_count <= 1 && !c->sparse &&
-                   !o.wait_limit_ns;   // (a limit of its waits is asked of the kernels that wait)
+                   (!o.wait_limit_ns || o.wait_limit_ns >= kDefaultLimitNs);   // (a shorter limit is asked of the
+                                                                               // kernels that wait)
     c->ap_lanes = (int)o.grid_lanes;
     c->ap_default = (o.lanes == 0 || o.lanes == 64) && (o.grid_lanes == 0 || o.grid_lanes == 128) && !o.blocks &&
                     (o.threads == 0 || o.threads == 512) && !o.heavy_words && (o.pull_div == 0 || o.pull_div == 32) &&
