@@ -2118,6 +2118,9 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
     bstat_init(s_bst);
     // an earlier launch of this run met a narrow wave: the per-CTA waves take the rest
     if (p.light && vload(p.light)) return;
+    // (trace: a run's launches number their waves on from one another's; the counter
+    // grows only when a launch ends)
+    const u32 wave0 = p.trace ? (u32)vload(&p.stats[ST_WAVES]) : 0;
     if (leader) {
         __syncthreads();   // s_thr, s_bst
         pick_wave(p, L, n_end, s_thr, s_bst, &st.mvis);
@@ -2197,7 +2200,7 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
                 const u32 cnt = d ? vload(&p.glist_n[cur]) : 0u;
                 const u64 arcs = d ? vload(&p.garc[cur]) : 0ull;
                 const bool pull = d && pull_wanted(p, W, arcs, s_minnd);
-                trace_record(p, TR_GRID_LEVEL, wave, d, cnt, alive | ((u64)pull << 16) | (arcs << 20), global_ns());
+                trace_record(p, TR_GRID_LEVEL, wave0 + wave, d, cnt, alive | ((u64)pull << 16) | (arcs << 20), global_ns());
             }
             if (d == 0) source_prefix<THREADS>(G, s_src, s_alive32, L, s_pre, s_beg, s_wsum);
             const u32 par = d & 1;
@@ -2341,7 +2344,7 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
         for (u32 i = blockIdx.x * THREADS + tid; i < nlog; i += gridDim.x * THREADS) clear_word<1>(S, __ldcg(&S.clog[i]));
         if (leader && tid == 0) bstat_add(s_bst, ST_CLEARED, nlog);
         if (!(ok = grid_sync(p.bar, gridDim.x, p.barrier_limit_ns, p.err))) break;
-        if (leader && tid == 0) trace_record(p, TR_GRID_WAVE, wave, d, nlog, wave_entries, global_ns());
+        if (leader && tid == 0) trace_record(p, TR_GRID_WAVE, wave0 + wave, d, nlog, wave_entries, global_ns());
         if (leader) {   // reset per-wave counters and advance the queue
             for (u32 i = tid; i < 2 * kCntParity; i += THREADS) p.gcnt[i] = 0;
             if (tid == 0) {
