@@ -2028,20 +2028,23 @@ __device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, co
         const u32 pos = base + tid;
         const bool have = pos < n_end;
         bool keep = have, done = false;
-        u32 v = 0, deg = 0;
+        u32 v = 0, scanned = 0;   // arcs of level 0, where the source passes its test
         if (have) {
             v = __ldg(&p.sources[pos]);
             if (p.pick && thr.valid) {
-                deg = p.walks.c[1][v];
+                const u32 deg = p.walks.c[1][v];
                 const u32 c2 = p.walks.c[2][v], xlo = __ldg(&p.g.xlo[v]), xhi = __ldg(&p.g.xhi[v]);
                 if (deg == 0) {
                     keep = !ranks_before(thr.N, thr.F, thr.id, 0, 1, v);
                     done = !keep;
                 } else {
                     const u32 two = c2 + (p.undirected && !p.footnote && c2 != kWalkMany ? deg : 0u);
-                    keep = !bfscut_stops(0, deg, 0, 1, xlo, xhi, v, thr) &&
-                           !bfscut_stops(deg, two, 1, 1 + deg, xlo, xhi, v, thr) &&
-                           !(use > 2 && walk_stops(p.walks, use, v, xlo, xhi, thr));
+                    keep = !bfscut_stops(0, deg, 0, 1, xlo, xhi, v, thr);
+                    if (keep) {
+                        scanned = deg;
+                        keep = !bfscut_stops(deg, two, 1, 1 + deg, xlo, xhi, v, thr) &&
+                               !(use > 2 && walk_stops(p.walks, use, v, xlo, xhi, thr));
+                    }
                 }
             }
         }
@@ -2061,7 +2064,7 @@ __device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, co
         cnt = cnt + total < L ? cnt + total : L;
         if (have && !keep && pos < base) {
             bstat_add(bst, done ? ST_COMPLETED : ST_CUT, 1);
-            *mvis += deg;
+            *mvis += scanned;
         }
         __syncthreads();
     }
