@@ -2013,8 +2013,7 @@ __device__ __forceinline__ bool pull_wanted(const WaveParams& p, int W, u64 farc
 // stop against the threshold by now (the prefilter ran against an earlier
 // one: on Barabasi-Albert n = 150,000, m = 3, top-100, 36,000 sources passed
 // it and 282 waves ran, 100 ms; with the picking 30 waves, 13.3 ms).
-__device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, const ThrCache& thr, BlockStats& bst,
-                                       u64* mvis) {
+__device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, const ThrCache& thr, BlockStats& bst) {
     __shared__ u32 s_cnt[32], s_last;
     const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
     __syncthreads();
@@ -2062,10 +2061,10 @@ __device__ __noinline__ void pick_wave(const WaveParams& p, u32 L, u32 n_end, co
         __syncthreads();
         base = s_last;
         cnt = cnt + total < L ? cnt + total : L;
-        if (have && !keep && pos < base) {
-            bstat_add(bst, done ? ST_COMPLETED : ST_CUT, 1);
-            *mvis += scanned;
-        }
+        const bool dropped = have && !keep && pos < base;
+        if (dropped) bstat_add(bst, done ? ST_COMPLETED : ST_CUT, 1);
+        scanned = __reduce_add_sync(0xffffffffu, dropped ? scanned : 0u);   // (other sources, other arcs: below m < 2^32)
+        if (lane == 0 && scanned) atomicAdd(&p.stats[ST_MVIS], (unsigned long long)scanned);
         __syncthreads();
     }
     if (tid == 0) {
@@ -2084,6 +2083,7 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
     __shared__ u32 s_cg[L], s_cs[L];
     __shared__ u32 s_alive32[2 * W];
     __shared__ u32 s_nc, s_base;
+    __shared__ u32 s_wave0;   // waves of the run's earlier launches (thread 0's, in shared memory: registers are short)
     __shared__ u32 s_minnd;   // fewest vertices a live lane has reached (push or pull)
     __shared__ u32 s_pgam[L]; // each lane's gamma of the frontier being expanded (m_vis of a pulled level)
     __shared__ ThrCache s_thr;
@@ -2123,10 +2123,10 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
     if (p.light && vload(p.light)) return;
     // (trace: a run's launches number their waves on from one another's; the counter
     // grows only when a launch ends)
-    const u32 wave0 = p.trace ? (u32)vload(&p.stats[ST_WAVES]) : 0;
+    if (p.trace && leader && tid == 0) s_wave0 = (u32)vload(&p.stats[ST_WAVES]);
     if (leader) {
         __syncthreads();   // s_thr, s_bst
-        pick_wave(p, L, n_end, s_thr, s_bst, &st.mvis);
+        pick_wave(p, L, n_end, s_thr, s_bst);
     }
     bool ok = grid_sync(p.bar, gridDim.x, p.barrier_limit_ns, p.err);
 
@@ -2203,7 +2203,7 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
                 const u32 cnt = d ? vload(&p.glist_n[cur]) : 0u;
                 const u64 arcs = d ? vload(&p.garc[cur]) : 0ull;
                 const bool pull = d && pull_wanted(p, W, arcs, s_minnd);
-                trace_record(p, TR_GRID_LEVEL, wave0 + wave, d, cnt, alive | ((u64)pull << 16) | (arcs << 20), global_ns());
+                trace_record(p, TR_GRID_LEVEL, s_wave0 + wave, d, cnt, alive | ((u64)pull << 16) | (arcs << 20), global_ns());
             }
             if (d == 0) source_prefix<THREADS>(G, s_src, s_alive32, L, s_pre, s_beg, s_wsum);
             const u32 par = d & 1;
@@ -2347,7 +2347,7 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
         for (u32 i = blockIdx.x * THREADS + tid; i < nlog; i += gridDim.x * THREADS) clear_word<1>(S, __ldcg(&S.clog[i]));
         if (leader && tid == 0) bstat_add(s_bst, ST_CLEARED, nlog);
         if (!(ok = grid_sync(p.bar, gridDim.x, p.barrier_limit_ns, p.err))) break;
-        if (leader && tid == 0) trace_record(p, TR_GRID_WAVE, wave0 + wave, d, nlog, wave_entries, global_ns());
+        if (p.trace && leader && tid == 0) trace_record(p, TR_GRID_WAVE, s_wave0 + wave, d, nlog, wave_entries, global_ns());
         if (leader) {   // reset per-wave counters and advance the queue
             for (u32 i = tid; i < 2 * kCntParity; i += THREADS) p.gcnt[i] = 0;
             if (tid == 0) {
@@ -2367,7 +2367,7 @@ __global__ void __launch_bounds__(THREADS, BCM_GRID_MIN_BLOCKS) k_wave_grid(Wave
             if (light) {
                 if (tid == 0 && p.light) vstore(p.light, 1u);
             } else if (wave + 1 < p.max_grid_waves) {
-                pick_wave(p, L, n_end, s_thr, s_bst, &st.mvis);
+                pick_wave(p, L, n_end, s_thr, s_bst);
             }
         }
         if (!(ok = grid_sync(p.bar, gridDim.x, p.barrier_limit_ns, p.err))) break;
