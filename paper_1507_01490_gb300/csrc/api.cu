@@ -729,6 +729,7 @@ bcm_status preprocess(bcm_graph* g, double* ms, bool topk = false) {
         const bool walks = topk && n >= 9728 && (g->directed || g->max_deg > kSparseMaxDeg) && ensure_walk_counts(g);
         Walks K{};
         K.c[1] = g->d_walk;
+        K.max_deg = g->max_deg;
         K.c[2] = (uint32_t*)((char*)g->d_walk + nb);
         K.heavy_n = (uint32_t*)(d_simple + 16);
         K.heavy = (uint32_t*)(d_scr2 + dos + scs + 256);
@@ -1001,6 +1002,7 @@ Walks carve_walks(bcm_graph* g) {
     K.heavy_n = g->d_aux->walk_heavy_n;
     K.want = &g->d_aux->walk_want;
     K.off = 0;
+    K.max_deg = g->max_deg;
     return K;
 }
 

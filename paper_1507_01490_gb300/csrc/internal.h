@@ -84,6 +84,7 @@ struct Walks {
     uint32_t* heavy_n;              // [kWalkLevels + 1]
     uint32_t* want;                 // the last c[j] there is (at least 2)
     uint32_t off;                   // no more than c[2]
+    uint32_t max_deg;               // the graph's longest row
 };
 
 struct WaveParams {

@@ -1194,8 +1194,13 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+__global__ void __launch_bounds__(512) k_walk_heavy(GraphDev G, Walks K, int j, bool undirected) {
+    if (j > 2 && (u32)j > *K.want) return;
+    walk_heavy<true>(G, K, j, undirected, kWalkLong);
+}
+
 __global__ void __cluster_dims__(kWalkCluster, 1, 1) __launch_bounds__(512)
-k_walk_heavy(GraphDev G, Walks K, int j, bool undirected) {
+k_walk_long(GraphDev G, Walks K, int j, bool undirected) {
     if (j > 2 && (u32)j > *K.want) return;
     walk_heavy<true>(G, K, j, undirected, kWalkLong);
     __shared__ unsigned long long s_part;
@@ -1425,13 +1430,19 @@ int launch_refilter(const WaveParams& p, const Walks& K, bool undirected, uint32
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// (a launch in clusters starts later, so it is for the graphs that have such rows)
+static void launch_walk_heavy(const GraphDev& G, const Walks& K, int j, bool undirected, cudaStream_t s) {
+    if (K.max_deg > kWalkLong) k_walk_long<<<152 * 4, 512, 0, s>>>(G, K, j, undirected);
+    else k_walk_heavy<<<152 * 4, 512, 0, s>>>(G, K, j, undirected);
+}
+
 int launch_prefilter(const WaveParams& p, const Walks& K, bool undirected, uint32_t* out, uint32_t* out_n,
                      cudaStream_t s) {
     if (p.g.n <= kWalkSmall) return launch_filter_small(p, K, undirected, true, out, out_n, s);
     const unsigned b = (p.g.n + 255) / 256 < 152 * 8 ? (p.g.n + 255) / 256 : 152 * 8;
     for (int j = 3; j <= kWalkLevels; ++j) {
         k_walk_sum<<<b, 256, 0, s>>>(p.g, K, j, undirected);
-        k_walk_heavy<<<152 * 4, 512, 0, s>>>(p.g, K, j, undirected);
+        launch_walk_heavy(p.g, K, j, undirected, s);
     }
     note_launch(2 * (kWalkLevels - 2));
     return launch_refilter(p, K, undirected, out, out_n, s);
@@ -1446,7 +1457,7 @@ int launch_walk_base(const uint32_t* rp, const uint32_t* col, uint32_t n, const 
     const unsigned b = (n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8;
     k_walk_degree<<<b, 256, 0, s>>>(G, K.c[1], K.heavy_n);
     k_walk_sum<<<b, 256, 0, s>>>(G, K, 2, undirected);
-    k_walk_heavy<<<152 * 4, 512, 0, s>>>(G, K, 2, undirected);
+    launch_walk_heavy(G, K, 2, undirected, s);
     note_launch(3);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
