@@ -1034,8 +1034,9 @@ __device__ __noinline__ void flush_completions(const WaveParams& p, const u32* c
 // is summed where that distance is above 2.75, c_4 above 3.75 (Chung-Lu and
 // R-MAT, 2.1 to 2.6, pay for neither).
 //
-//   k_walk_degree, k_walk_sum, k_walk_heavy   c_1; c_{j+1} from c_j.  c_1 and
-//                 c_2 belong to the graph's preprocessing
+//   k_walk_degree, k_walk_sum, k_walk_heavy (k_walk_long)   c_1; c_{j+1} from c_j.  c_1 and
+//                 c_2 are made beside the graph's preprocessing, or by the first
+//                 run that wants them
 //   k_prefilter   32 consecutive positions of the source list per warp: the
 //                 stopping rule at levels 0 and 1 as a wave would apply it, then
 //                 the bounds; one bit per position says that it stays

@@ -64,7 +64,13 @@ inline uint32_t spread_step(uint32_t count) {
 
 // Is that shape worth taking?  A large graph whose planes leave L2 (`budget`)
 // with most SMs idle stays on the kernels that search from sources; so does one
-// that no shape fits.
+// that no shape fits.  With 130 MB on 152 SMs the line lies at about 284,000
+// vertices.  Farness of every vertex, grid-wide kernel -> all pairs: Chung-Lu of
+// 100,000 vertices and 16 arcs each 307 -> 43 ms, 200,000 687 -> 293, 283,000
+// 987 -> 412, R-MAT 2^18 and 12 arcs 563 -> 455; deep graphs too (a grid-wide
+// level costs two barriers of the whole grid for 128 sources): a directed path of
+// 8,000 4,164 -> 43, paths of 30 in 280,000 1,020 -> 607, a ring of 131,072 and 40
+// arcs 279 -> 217 s.
 inline bool allpairs_fits(uint32_t n, int sms, size_t budget, int lanes, int* W, int* C, int* clusters) {
     const int busy = allpairs_shape(n, sms, budget, lanes, W, C, clusters);
     if (busy <= 0) return false;
