@@ -107,8 +107,9 @@ typedef enum {
  * on the all-pairs kernel (targets as lanes) where the bit planes of enough
  * waves for three quarters of the SMs fit 130 MB, about L2's size (up to about
  * 284,000 vertices), and top-k runs of small graphs with no launch parameter set take their answer
- * from every vertex's farness by that kernel (n <= 16,384 and n m below 2^30,
- * or 2^32 for k > 32 or n < 9,728).  Levels of grid waves
+ * from every vertex's farness by that kernel (n <= 16,384 and n m at most 2^32;
+ * from n = 9,728 on, k <= 32 only on undirected graphs, n m at most 2^30 k / 20,
+ * or 2^30 if m <= 33/16 n).  Levels of grid waves
  * run by push (each frontier vertex
  * sets its lanes' bits in its out-neighbours) or, when the frontier's arcs
  * are a large share of the graph's, by pull (each vertex with lanes still

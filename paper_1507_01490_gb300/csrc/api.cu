@@ -588,10 +588,16 @@ constexpr size_t kApLanesBytes = 48 * sizeof(uint32_t);
 // 64): complete searches of a small graph from every vertex are cheaper than
 // one wave that sets a threshold and the tests behind it.  BA 2000, m = 3,
 // top-10: 0.41 ms with the seed wave, 0.14 here; BA 8000, m = 8, top-100 5.9,
-// 0.37.  With grid-wide waves (n >= 9,728) only a long list, which leaves the
-// first wave's threshold weak, pays for more (BA 16,000, m = 4: top-10 0.28 ms
-// on the grid, top-100 3.0; here 0.7).
+// 0.37.  With grid-wide waves (n >= 9,728) a long list, which leaves the first
+// wave's threshold weak, pays for as much (BA 16,000, m = 4: top-10 0.28 ms on
+// the grid, top-100 3.0; here 0.7).  A shorter one pays in proportion to its
+// length, kApShortWords an entry -- undirected Chung-Lu 12,500 vertices, mean
+// degree 4, top-1 0.29 ms on the grid, top-10 0.33, top-32 1.5, here 0.75 -- or
+// on a graph that is hardly more than a tree, whose distances no bound foresees
+// (BA 16,300, m = 1, top-1 to 10 1.2 to 5.8, here 1.5).  On digraphs it does not
+// (R-MAT 2^14, 4 arcs a vertex, top-1 0.29 on the grid, top-32 1.3; here 1.05).
 constexpr uint64_t kApTopkWords = 1ull << 24, kApTopkWordsMost = 1ull << 26;
+constexpr uint64_t kApShortWords = kApTopkWords / 20;
 constexpr uint32_t kApLongList = 32;
 constexpr uint64_t kApMostArcs = 1ull << 28;   // its copy of the rows: 1 GB
 // Grid-wide waves take 256 lanes while this many sources are queued, 128 after
@@ -606,7 +612,11 @@ bool all_pairs_shape(bcm_graph* g, const Cfg& c, bool exhaustive, uint32_t k, Ap
     if (!c.all_pairs || g->n < 2 || g->m > kApMostArcs) return false;
     if (!exhaustive) {
         const bool small = (uint64_t)g->n * c.grid_W < c.heavy_words;
-        const uint64_t most = small || k > kApLongList ? kApTopkWordsMost : kApTopkWords;
+        const bool tree = g->m <= 2 * (uint64_t)g->n + g->n / 16;
+        const uint64_t most = small || k > kApLongList          ? kApTopkWordsMost
+                              : g->directed                     ? 0
+                              : tree || k * kApShortWords > kApTopkWords ? kApTopkWords
+                                                                : k * kApShortWords;
         if (!c.ap_default || g->n > kAllPairsTopkN || (uint64_t)g->n * g->m / 64 > most) return false;
     }
     return allpairs_fits(g->n, g->sms, kAllPairsL2, exhaustive ? c.ap_lanes : 0, &a->W, &a->C, &a->clusters);
