@@ -136,7 +136,7 @@ typedef struct {
                                  (W = grid_lanes/64; 0 = default, 32) and at least a quarter of the
                                  pull's estimated cost, n/4 + (n - n_min) m/n, n_min the fewest vertices
                                  a live source has reached (so a lattice's thin frontiers stay push) */
-    uint32_t defer_words;     /* a per-CTA wave about to expand a level of this many words (or of 8x
+    uint32_t defer_words;     /* a per-CTA wave about to expand a level of this many words (or of 4x
                                  as many out-arcs) stops and hands its live sources to a second
                                  grid-wide pass, which runs them from the start; 0 = default
                                  (heavy_words) */

@@ -1464,6 +1464,14 @@ int launch_walk_base(const uint32_t* rp, const uint32_t* col, uint32_t n, const 
 }
 
 // --------------------------------------------------------- per-CTA waves
+// A wave hands its sources over before a level of this many out-arcs a word of
+// defer_words, too: 155,000 (8) took one CTA 1.2 to 1.5 ms, more than the grid
+// takes for ten such waves.  Resident R-MAT 2^15, 10 arcs a vertex, top-10,
+// whose waves lie at that line: 8 2.20 ms, 4 1.03; 5 arcs 2.42 and 0.62;
+// Chung-Lu 20,000, mean degree 12, top-100 unchanged (0.49).  At 2 and 1
+// Barabasi-Albert 700,000, m = 2, top-10 is slower (10.9, 10.1 and 14.5 ms).
+constexpr u64 kDeferArcs = 4;
+
 template <int W, int THREADS>
 __global__ void __launch_bounds__(THREADS, (1024 / THREADS) > 0 ? (1024 / THREADS) : 1) k_wave_cta(WaveParams p) {
     constexpr int L = 64 * W;
@@ -1576,7 +1584,7 @@ __global__ void __launch_bounds__(THREADS, (1024 / THREADS) > 0 ? (1024 / THREAD
             for (int i = 0; i < 2 * W; ++i) any |= s_alive32[i];
             if (!any) break;
 
-            if (d > 0 && p.defer_words && (s_ln[cur] >= p.defer_words || s_arcs[cur] >= 8ull * p.defer_words)) {
+            if (d > 0 && p.defer_words && (s_ln[cur] >= p.defer_words || s_arcs[cur] >= kDeferArcs * p.defer_words)) {
                 // a level too wide for one CTA is next (many frontier words,
                 // or few with very many out-arcs): the live sources go to the
                 // grid-wide pass, which runs them again from the start; the
