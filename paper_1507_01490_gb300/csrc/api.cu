@@ -301,6 +301,7 @@ struct Aux : RunOut {
     uint32_t walk_left[2];   // sources left by the prefilter, and by the second one
     uint32_t walk_heavy_n[kWalkLevels + 1];
     uint32_t walk_want;
+    uint32_t walk_probe[3];
     uint32_t head3;       // queue head of the waves over the sources left
     uint32_t head4;       // queue head of the per-CTA waves after the second prefilter
     uint32_t wave_src[256];   // the grid-wide kernel's next wave
@@ -1011,6 +1012,7 @@ Walks carve_walks(bcm_graph* g) {
     K.keep = (uint32_t*)p;
     K.heavy_n = g->d_aux->walk_heavy_n;
     K.want = &g->d_aux->walk_want;
+    K.probe = g->d_aux->walk_probe;
     K.off = 0;
     K.max_deg = g->max_deg;
     return K;

@@ -83,6 +83,7 @@ struct Walks {
     uint32_t* keep;                 // which positions of the source list stay
     uint32_t* heavy_n;              // [kWalkLevels + 1]
     uint32_t* want;                 // the last c[j] there is (at least 2)
+    uint32_t* probe;                // [3] zeroed: k_walk_probe's counts, blocks done
     uint32_t off;                   // no more than c[2]
     uint32_t max_deg;               // the graph's longest row
 };

@@ -1037,6 +1037,7 @@ __device__ __noinline__ void flush_completions(const WaveParams& p, const u32* c
 //   k_walk_degree, k_walk_sum, k_walk_heavy (k_walk_long)   c_1; c_{j+1} from c_j.  c_1 and
 //                 c_2 are made beside the graph's preprocessing, or by the first
 //                 run that wants them
+//   k_walk_probe  are c_3 and c_4 worth their passes (graphs above 65,536 vertices)
 //   k_prefilter   32 consecutive positions of the source list per warp: the
 //                 stopping rule at levels 0 and 1 as a wave would apply it, then
 //                 the bounds; one bit per position says that it stays
@@ -1233,6 +1234,49 @@ k_walk_long(GraphDev G, Walks K, int j, bool undirected) {
     }
 }
 
+// Counts beyond c_2 are not summed where the tests at levels 0 and 1 leave
+// about a wave: c_3 is a pass over all arcs (BA 700,000, m = 8, top-10: the whole
+// call 0.77 ms without walk bounds, 1.17 with c_3, 0.77 so).  Of large graphs
+// kProbe sources spread over the queue are tested, and its next kProbeNext: a
+// leaf beside a hub can outlast vertices of higher degree, so none of the
+// former may stay, and fewer than kProbeFew of the latter.
+constexpr u32 kProbe = 9728, kProbeNext = 512, kProbeFew = 128;
+
+__device__ __forceinline__ bool base_stays(const WaveParams& p, const Walks& K, bool undirected, u32 v,
+                                           const ThrCache& t) {
+    const u32 deg = __ldcg(&K.c[1][v]), c2 = __ldcg(&K.c[2][v]), xlo = __ldg(&p.g.xlo[v]);
+    const u32 xhi = undirected ? xlo : __ldg(&p.g.xhi[v]);
+    if (deg == 0) return !ranks_before(t.N, t.F, t.id, 0, 1, v);
+    const u32 two = c2 + (undirected && !p.footnote && c2 != kWalkMany ? deg : 0u);
+    return !bfscut_stops(0, deg, 0, 1, xlo, xhi, v, t) && !bfscut_stops(deg, two, 1, 1 + deg, xlo, xhi, v, t);
+}
+
+__global__ void __launch_bounds__(512) k_walk_probe(WaveParams p, Walks K, bool undirected) {
+    if (*K.want <= 2) return;
+    __shared__ ThrCache s_thr;
+    __shared__ u32 s_begin;
+    if (threadIdx.x == 0) {
+        s_thr.valid = 0; s_thr.N = 0; s_thr.F = 1; s_thr.id = 0;
+        read_thresholds(p.topk, s_thr);
+        s_begin = vload(p.head);
+    }
+    __syncthreads();
+    const u32 n_end = p.n_end_dev ? vload(p.n_end_dev) : p.n_end, begin = s_begin < n_end ? s_begin : n_end;
+    const bool next = blockIdx.x == gridDim.x - 1;   // the last block: the sources next in the queue
+    const u32 i = next ? threadIdx.x : blockIdx.x * 512 + threadIdx.x;
+    const u64 pos = next ? (u64)begin + i : begin + (u64)(n_end - begin) * i / kProbe;
+    const bool have = pos < n_end && (next || i < kProbe);
+    const bool stays = have && (!s_thr.valid || base_stays(p, K, undirected, __ldg(&p.sources[pos]), s_thr));
+    const u32 m = __ballot_sync(0xffffffffu, stays);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(&K.probe[next ? 1 : 0], __popc(m));
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&K.probe[2], 1u) == gridDim.x - 1) {
+        __threadfence();
+        if (vload(&K.probe[0]) == 0 && vload(&K.probe[1]) < kProbeFew) *K.want = 2;
+    }
+}
+
 // Does one of the bounds with J = 2 .. last stop v?  Each J is a line in x =
 // r(v), so the two ends of its range decide (Lemma 2's argument).
 __device__ __forceinline__ bool walk_stops(const Walks& K, int last, u32 v, u32 xlo, u32 xhi, const ThrCache& t) {
@@ -1396,7 +1440,20 @@ k_filter_small(WaveParams p, Walks K, bool undirected, bool sums, u32* out, u32*
     }
     bstat_init(s_bst);
     cluster_barrier();
-    const u32 want = __ldcg(K.want);
+    u32 want = __ldcg(K.want);
+    if (sums && want > 2) {   // every source here (no more than eight a thread)
+        const u32 end = p.n_end_dev ? vload(p.n_end_dev) : p.n_end;
+        u32 left = 0;
+        for (size_t pos = s_begin + tid; pos < end; pos += stride)
+            left += !s_thr.valid || base_stays(p, K, undirected, __ldg(&p.sources[pos]), s_thr);
+        left = __reduce_add_sync(0xffffffffu, left);
+        if ((threadIdx.x & 31) == 0 && left) atomicAdd(&K.probe[1], left);
+        cluster_barrier();
+        if (__ldcg(&K.probe[1]) < kProbeFew) {   // (the same in every CTA)
+            want = 2;
+            if (tid == 0) *K.want = 2;   // for the later launches; every CTA has read it
+        }
+    }
     for (u32 j = 3; sums && j <= want; ++j) {
         walk_sums<false>(p.g, K, (int)j, undirected, tid, stride);
         cluster_barrier();
@@ -1441,6 +1498,8 @@ int launch_prefilter(const WaveParams& p, const Walks& K, bool undirected, uint3
                      cudaStream_t s) {
     if (p.g.n <= kWalkSmall) return launch_filter_small(p, K, undirected, true, out, out_n, s);
     const unsigned b = (p.g.n + 255) / 256 < 152 * 8 ? (p.g.n + 255) / 256 : 152 * 8;
+    k_walk_probe<<<kProbe / 512 + 1, 512, 0, s>>>(p, K, undirected);
+    note_launch();
     for (int j = 3; j <= kWalkLevels; ++j) {
         k_walk_sum<<<b, 256, 0, s>>>(p.g, K, j, undirected);
         launch_walk_heavy(p.g, K, j, undirected, s);
