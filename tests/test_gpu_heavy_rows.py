@@ -59,12 +59,10 @@ def test_more_rows_than_the_list_holds(B, gen, orc):
     assert count == nc and np.array_equal(lo, al) and np.array_equal(hi, om)
 
 
-def test_one_row_of_a_million(B, gen):
-    """Its time: shared by the whole grid it took 2.3 ms more or less, in four pieces 3.4; the mean of both is the
-    bound, on the best of 20."""
+def _scc_time(B, gen, n, src, dst):
+    """The best of 20 whole calls (handle, SCCs and bounds, release), and alpha."""
     import torch
-    n, m = 1200000, 1000000
-    g = gen.csr_from_arcs(n, np.zeros(m, np.int64), np.arange(1, m + 1), directed=True, name="dstar")
+    g = gen.csr_from_arcs(n, src, dst, directed=True, name="rows")
     rp = torch.from_numpy(g.row_ptr.view(np.int64)).cuda()
     col = torch.from_numpy(g.col.view(np.int32)).cuda()
     out = [torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(3)]
@@ -75,6 +73,14 @@ def test_one_row_of_a_million(B, gen):
         with B.BcmGraph(rp, col, n, True, on_device=True) as h:
             assert B.bcm_scc_bounds(h.h, *out, out_on_device=True) == n
         best = min(best, (time.perf_counter() - t0) * 1e3)
-    lo = out[1].cpu().numpy()
+    return best, out[1].cpu().numpy()
+
+
+def test_one_row_of_a_million(B, gen):
+    """Its time against that of the same arcs in rows of 2,000, which are short: the whole grid on the row took as long,
+    four blocks on it half as long again, so a quarter more is the bound."""
+    n, m = 1200000, 1000000
+    one, lo = _scc_time(B, gen, n, np.zeros(m, np.int64), np.arange(1, m + 1))
     assert lo[0] == m + 1 and (lo[1:] == 1).all()   # (the first of the largest SCCs: its reach is measured)
-    assert best < 2.85, best
+    many, _ = _scc_time(B, gen, n, np.repeat(np.arange(500), 2000), np.arange(500, m + 500))
+    assert one < 1.25 * many, (one, many)
